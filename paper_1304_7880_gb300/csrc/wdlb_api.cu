@@ -260,6 +260,21 @@ wdlb_status check_status_word(wdlb_ctx *ctx)
     return WDLB_OK;
 }
 
+// Whether the generic shell kernel splits a node's pairs over four warps (one
+// fourth of the sum each, then one warp for the collision).  Splitting pays
+// wherever the sums outweigh the collision, which three of the four warps sit
+// out: always on the full shells (31 pairs at sigma 2 and more), and on any
+// shell while the lattice leaves SMs without a block of 256 nodes.  Shell
+// kernel, unsplit against split, us: sigma 8 full FP32 256.6 / 36.9 on 4 096
+// nodes, 2 321 / 1 500 on 96^3; sigma 3 full (PY) 325 / 291 on 96^3; sigma 4
+// full FP64 585 / 92 on 4 096 nodes, 1 697 / 1 531 on 48^3.  Sigma 8 compact
+// (21 pairs): 20.6 / 11.9 on 16 384 nodes, 20.5 / 20.6 on 36 864, 178 / 228 on
+// 96^3; in FP64 at sigma 4 156 / 109 and 156 / 166 on the first two.
+int split_shell(int npair, long long N)
+{
+    return npair >= 31 || N <= 24576 ? 1 : 0;
+}
+
 void set_params(wdlb_ctx *ctx)
 {
     KParams &p = ctx->kp;
@@ -292,6 +307,9 @@ void set_params(wdlb_ctx *ctx)
     const double s2 = 2.0 * ctx->sigma;
     p.s2 = (std::fabs(s2 - std::round(s2)) < 1e-12) ? (int)std::lround(s2) : 0;
     p.tiled = 0;
+    p.shell_r = 0;
+    for (int c : ctx->tab.shell) p.shell_r = std::max(p.shell_r, std::abs(c));
+    p.split = split_shell(p.nshell / 2, ctx->N);
     p.ball_r = 0;
     for (size_t m = 0; m < ctx->tab.ball.size(); m++) p.ball_r = std::max(p.ball_r, std::abs(ctx->tab.ball[m]));
     const size_t tsize = ctx->opt.storage == WDLB_STORE_F64 ? sizeof(double) : sizeof(float);
@@ -366,6 +384,7 @@ cudaError_t upload_step_tables(wdlb_ctx *ctx)
     G.closure = p.closure;
     G.tile = p.tiled ? p.tile : -1;
     G.rule = p.shell_rule;
+    G.split = p.tiled ? 0 : p.split;
     G.items = dit + items.size();
     if (p.tiled)
         bricks(tile_depth(p.tile));
@@ -1270,11 +1289,11 @@ wdlb_status batch_build(wdlb_batch *b)
     std::vector<BatchItem> node_items, ball_items, ball_node_items;
     size_t ball_smem = 0;
     struct Key {
-        int s2, walls, tiled, closure, tile, rule;
+        int s2, walls, tiled, closure, tile, rule, split;
         bool operator<(const Key &o) const
         {
-            return std::make_tuple(s2, walls, tiled, closure, tile, rule) <
-                   std::make_tuple(o.s2, o.walls, o.tiled, o.closure, o.tile, o.rule);
+            return std::make_tuple(s2, walls, tiled, closure, tile, rule, split) <
+                   std::make_tuple(o.s2, o.walls, o.tiled, o.closure, o.tile, o.rule, o.split);
         }
     };
     std::map<Key, std::vector<BatchItem>> groups;
@@ -1299,7 +1318,7 @@ wdlb_status batch_build(wdlb_batch *b)
             for (int k = 0; k < (N + 255) / 256; k++) ball_node_items.push_back(BatchItem{s, k, 0, 0});
         }
         Key key{c->kp.tiled ? c->kp.s2 : 0, c->walls, c->kp.tiled, c->kp.closure, c->kp.tiled ? c->kp.tile : -1,
-                c->kp.shell_rule};
+                c->kp.shell_rule, c->kp.tiled ? 0 : c->kp.split};
         auto &g = groups[key];
         if (c->kp.tiled) {
             const int depth = tile_depth(c->kp.tile);
@@ -1346,6 +1365,7 @@ wdlb_status batch_build(wdlb_batch *b)
         G.closure = g.first.closure;
         G.tile = g.first.tile;
         G.rule = g.first.rule;
+        G.split = g.first.split;
         G.items = b->d_items + all.size();
         G.nitems = (int)g.second.size();
         all.insert(all.end(), g.second.begin(), g.second.end());

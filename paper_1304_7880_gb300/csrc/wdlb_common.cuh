@@ -56,6 +56,8 @@ struct KParams {
     int shell_rule;          // 0: full shell, uniform weight wshell; 1: compact shell,
                              // per-vector weights in shell_k[m].w (wshell = 1)
     int tma;                 // 1: the tiled shell kernel stages interior bricks' tiles by TMA
+    int shell_r;             // largest |component| of a shell vector (at most kMaxShellR)
+    int split;               // 1: the generic shell kernel splits a node's pairs over four warps
     int wait_limit;          // polls of an mbarrier wait before it gives up (status bit 4)
     const void *tmaps;       // device tensor maps of nu and hb for the TMA tile (64-byte aligned)
     double g[3];             // external acceleration
@@ -108,6 +110,8 @@ template <>
 __device__ __forceinline__ double prm<double>(double d, float) { return d; }
 template <>
 __device__ __forceinline__ float prm<float>(double, float f) { return f; }
+
+constexpr int kMaxShellR = 8;    // floor(sigma + 1/2) for sigma <= 8
 
 // Tiled ball sum: an 8 x 8 x 8 brick of nodes per block with a halo of
 // ball_r, the brick's n - n_off and the ball's offsets in shared memory.

@@ -816,6 +816,94 @@ __device__ __forceinline__ void shell_body(const KParams &p, const KBufs<S, type
                                            me.x, target_dn);
 }
 
+// ---------------------------------------------------------------------------
+// Split form of shell_body: a block of kSplit warps serves 32 nodes, lane l of
+// every warp the same node, and warp k sums the pairs k, k + kSplit, ... of the
+// table; warp 0 adds the partial sums in warp order and runs the collision.
+// Unsplit, the kernel is bound by each warp's own chain of loads and sums (FP32:
+// 381 pairs at sigma 8, ~400 instructions each) or by the FP64 pipe of the few
+// SMs that hold a block (two lanes a clock), so a lattice of few blocks leaves
+// most of the chip idle; four warps for an eighth of the nodes spread the same
+// sums.  Wrapped neighbour coordinates are formed once per node and shell
+// component (2 R + 1 per axis) into shared memory; beyond a wall they point at
+// the solid plane z = 0, whose nu and hb hold the n = 0 state, so a neighbour's
+// index is the sum of three words with no test.  Shell kernel, before and now:
+// sigma 8 on 8 x 8 x 256 (FP32) 256.8 -> 39.5 us, the 8 x 8 x 41 slit in FP64
+// 547 -> 94 us, a 48^3 box in FP64 1 697 -> 1 531 us (bound by the FP64 pipe).
+// ---------------------------------------------------------------------------
+constexpr int kSplit = 4;
+
+template <class S, int CL, bool WALLS, bool WT, class A = typename Store<S>::T>
+__device__ __forceinline__ void shell_split_body(const KParams &p, const KBufs<S, typename Store<S>::T> &b, int node0)
+{
+    typedef typename Store<S>::T T;
+    constexpr int NACC = sizeof(ShellAcc<T>) / sizeof(T);
+    __shared__ int axis[3][2 * kMaxShellR + 1][32];
+    __shared__ T part[kSplit - 1][NACC][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nx = p.nx, ny = p.ny, nz = p.nz, R = p.shell_r;
+    const int i = min(node0 + lane, p.N - 1);
+    const int x = i % nx, y = (i / nx) % ny, z = i / (nx * ny);
+    const bool fluid = node0 + lane < p.N && !(WALLS && (z == 0 || z == nz - 1));
+    for (int k = wid; k <= 2 * R; k += kSplit) {
+        const int zz = z + k - R;
+        axis[0][k][lane] = wrap_coord(x + k - R, nx);
+        axis[1][k][lane] = nx * wrap_coord(y + k - R, ny);
+        axis[2][k][lane] = nx * ny * (WALLS ? (zz < 0 || zz >= nz ? 0 : zz) : wrap_coord(zz, nz));
+    }
+    __syncthreads();
+
+    const T noff = prm<T>(p.n_off, p.f_n_off), hoff = prm<T>(p.h_off, p.f_h_off);
+    const T hr = hoff + b.hb[i];
+    const V4<T> me = b.nu[i];
+    ShellAcc<T> a = {};
+    if (fluid && p.interactions) {
+        const T s0 = T(1) - hr - hoff;
+        const int npair = p.nshell >> 1;
+#pragma unroll 2
+        for (int m = wid; m < npair; m += kSplit) {
+            const int4 e = b.shell_e[2 * m];
+            const V4<T> k = b.shell_k[2 * m];
+            const int jp = axis[0][R + e.x][lane] + axis[1][R + e.y][lane] + axis[2][R + e.z][lane];
+            const int jm = axis[0][R - e.x][lane] + axis[1][R - e.y][lane] + axis[2][R - e.z][lane];
+            if (!in_bounds(jp, p.N, b.status) || !in_bounds(jm, p.N, b.status)) continue;
+            const V4<T> np = b.nu[jp], nm = b.nu[jm];
+            const T hp = b.hb[jp], hm = b.hb[jm];
+            T qp, qm, qd;
+            pair_weights<CL, T>(s0, noff, hp, np.x, hm, nm.x, qp, qm, qd);
+            if (WT) {
+                qp *= k.w;
+                qm *= k.w;
+                qd *= k.w;
+            }
+            accumulate_pair<T>(a, k.x, k.y, k.z, qp, qm, qd, np.y, np.z, np.w, nm.y, nm.z, nm.w, me.y, me.z, me.w);
+        }
+    }
+    T *acc = reinterpret_cast<T *>(&a);
+    if (wid > 0) {
+#pragma unroll
+        for (int c = 0; c < NACC; c++) part[wid - 1][c][lane] = acc[c];
+    }
+    __syncthreads();
+    if (wid > 0 || !fluid) return;
+#pragma unroll
+    for (int k = 0; k < kSplit - 1; k++)
+#pragma unroll
+        for (int c = 0; c < NACC; c++) acc[c] += part[k][c][lane];
+
+    T Cx = T(0), Cy = T(0), Cz = T(0), Axx = T(0), Ayy = T(0), Azz = T(0), Axy = T(0), Axz = T(0), Ayz = T(0);
+    T tsum = T(0);
+    if (p.interactions)
+        shell_forces<T>(p, a, noff + me.x, me.y, me.z, me.w, Cx, Cy, Cz, Axx, Ayy, Azz, Axy, Axz, Ayz, tsum);
+    const auto target_dn = [&](int, int dst) { return in_bounds(dst, p.N, b.status) ? b.nu[dst].x : T(0); };
+    if constexpr (is_dw<A>::value)
+        collide_push_dw<S, CL, WALLS>(p, b, i, x, y, z, hr, Cx, Cy, Cz, Axx, Ayy, Azz, Axy, Axz, Ayz, tsum, me.x,
+                                      target_dn);
+    else
+        collide_push<S, CL, WALLS, false>(p, b, i, x, y, z, hr, Cx, Cy, Cz, Axx, Ayy, Azz, Axy, Axz, Ayz, tsum, me.x,
+                                          target_dn);
+}
+
 template <class S, int CL, bool WALLS, bool FIELDS, bool WT>
 __global__ void __launch_bounds__(256) k_shell_collide(KParams p, KBufs<S, typename Store<S>::T> b)
 {

@@ -283,6 +283,16 @@ void kbufs_fill(const DevBufs &d, int cur, void *out)
     std::memcpy(out, &b, sizeof(b));
 }
 
+template <int CL, bool WALLS, bool WT>
+void launch_generic(const BatchLaunch &L, const KBufs<S, T> *B, const BatchGroup &G, cudaStream_t st)
+{
+    if (G.split)
+        k_step_shell_split<S, CL, WALLS, WT, A>
+            <<<G.nitems * kSplitBlocks, 32 * kSplit, 0, st>>>(L.params, B, G.items);
+    else
+        k_step_shell<S, CL, WALLS, WT, A><<<G.nitems, kThreads, 0, st>>>(L.params, B, G.items);
+}
+
 cudaError_t do_batch_step(const BatchLaunch &L, int parity, int part, int group, cudaStream_t st,
                           int64_t *launches)
 {
@@ -317,12 +327,12 @@ cudaError_t do_batch_step(const BatchLaunch &L, int parity, int part, int group,
             continue;
         }
 #endif
-#define WDLB_SB(CLV, WV)                                                                         \
-    do {                                                                                         \
-        if (G.rule)                                                                              \
-            k_step_shell<S, CLV, WV, true, A><<<G.nitems, kThreads, 0, st>>>(L.params, B, G.items);  \
-        else                                                                                     \
-            k_step_shell<S, CLV, WV, false, A><<<G.nitems, kThreads, 0, st>>>(L.params, B, G.items); \
+#define WDLB_SB(CLV, WV)                                          \
+    do {                                                          \
+        if (G.rule)                                               \
+            launch_generic<CLV, WV, true>(L, B, G, st);           \
+        else                                                      \
+            launch_generic<CLV, WV, false>(L, B, G, st);          \
     } while (0)
         if (G.walls) {
             if (G.closure == 0) WDLB_SB(0, true);
