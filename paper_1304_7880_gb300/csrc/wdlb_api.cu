@@ -54,6 +54,7 @@ struct Tables {
     std::vector<int> shell;   // 3 per vector, +e and -e adjacent
     std::vector<double> wvec; // weight of each shell vector
     double wshell = 0.0;      // uniform weight in the kernels (1 for the compact shell)
+    int ncouple = 0;          // mirror couples at the head of a full shell
 };
 
 struct Layout {
@@ -286,6 +287,7 @@ void set_params(wdlb_ctx *ctx)
     p.Npad = (int)ctx->Npad;
     p.nshell = (int)(ctx->tab.shell.size() / 3);
     p.nball = (int)(ctx->tab.ball.size() / 3);
+    p.ncouple = ctx->tab.ncouple;
     p.closure = ctx->opt.closure;
     p.shell_rule = ctx->opt.shell_rule;
     p.omega_mode = ctx->opt.omega_mode;
@@ -333,6 +335,22 @@ void drop_graphs(wdlb_ctx *ctx)
             cudaGraphExecDestroy(g);
             g = nullptr;
         }
+}
+
+// Shell groups take the roomy form where all of a step's blocks together leave
+// SMs without one (groups run side by side).
+void mark_roomy(BatchLaunch &L)
+{
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            n = 0;
+        return n;
+    }();
+    int blocks = 0;
+    for (int g = 0; g < L.ngroups; g++) blocks += L.groups[g].nitems;
+    for (int g = 0; g < L.ngroups; g++) L.groups[g].roomy = L.groups[g].tiled && blocks <= sms;
 }
 
 // One-slot step tables of a lattice stepped alone: its parameters, its
@@ -392,6 +410,7 @@ cudaError_t upload_step_tables(wdlb_ctx *ctx)
         blocks();
     G.nitems = (int)(items.size() - (G.items - dit));
     LL.ngroups = 1;
+    mark_roomy(LL);
     if (items.size() > L.nitems) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemcpyAsync(b + L.params, &p, sizeof(KParams), cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess)
@@ -644,6 +663,7 @@ wdlb_status wdlb_create(wdlb_lattice lat, double sigma, int32_t walls, double ta
     ctx->Npad = (ctx->N + 63) / 64 * 64;
     build_ball(sigma, ctx->tab.ball);
     build_shell_rule(sigma, o.shell_rule, ctx->tab.shell, ctx->tab.wvec);
+    if (o.shell_rule == WDLB_SHELL_FULL) ctx->tab.ncouple = order_couples(ctx->tab.shell);   // one weight for all
     ctx->tab.wshell = o.shell_rule == WDLB_SHELL_COMPACT ? 1.0 : ctx->tab.wvec[0];
     ctx->L = &launchers_for(o.storage, o.collision);
     set_params(ctx);
@@ -1370,6 +1390,7 @@ wdlb_status batch_build(wdlb_batch *b)
         G.nitems = (int)g.second.size();
         all.insert(all.end(), g.second.begin(), g.second.end());
     }
+    mark_roomy(L);
     cudaError_t e = cudaSuccess;
     // item counts per slot and phase for the persistent step
     b->flow = b->opt.persistent && b->L->flow_ok(L);

@@ -47,6 +47,7 @@ struct KParams {
     int nx, ny, nz, walls;   // walls: solid planes z = 0 and z = nz-1
     int N, Npad;             // node count, padded stride of per-node arrays
     int nshell, nball;
+    int ncouple;             // mirror couples at the head of the shell table (order_couples); 0: compact shell
     int closure, omega_mode, interactions;
     int s2;                  // 2 sigma if it is an integer, else 0 (selects a compiled shell)
     int tiled;               // 1: use the shared-memory tiled shell kernel

@@ -308,16 +308,22 @@ __device__ __forceinline__ void ball_brick_ct(const KParams &p, const V4<T> *nu,
 // ---------------------------------------------------------------------------
 // Pair weights of a (+e, -e) pair of the contact shell.  With
 // q = g2(chi_mid) n(r+e) (without the quadrature weight), chi_mid/2 =
-// hb(r) + hb(r+e), the weights are carried doubled, Q = 2q, which makes the
-// Carnahan-Starling value one multiply-add: 2 g2 = (1 + s)/s^3 with
-// s = 1 - chi_mid (Percus-Yevick: (3 - s)/s^2; closure one: 2).  s0 = 1 - h(r)
-// - h_off; dh, dn: deviations of the two neighbours.  Besides Q+ and Q- it
-// returns 2 (Q+ - Q-), formed from the deviations so that it is accurate
-// relative to itself (it is what the mean-field sum accumulates):
-//   2 (Q+ - Q-) = (G+ + G-)(dn+ - dn-) + (G+ - G-)(n+ + n-),   G = 2 g2,
-//   CS:  G+ - G- = (dh+ - dh-) [s+^2 + s-^2 + s+ s- (1 + s+ + s-)] / (s+^3 s-^3)
-//   PY:  G+ - G- = (dh+ - dh-) [3 (s+ + s-) - s+ s-] / (s+^2 s-^2)
-// (exact divided differences of the closures; s- - s+ = dh+ - dh-).
+// hb(r) + hb(r+e), the weights are carried doubled, Q = 2q, which drops the
+// factor 1/2 of the closures: with a = 1/s, s = 1 - chi_mid, G = 2 g2 is
+//   CS: a^2 + a^3    PY: 3 a^2 - a    closure one: 2.
+// s0 = 1 - h(r) - h_off; dh, dn: deviations of the two neighbours.  Besides Q+
+// and Q- it returns 2 (Q+ - Q-), formed from the deviations so that it is
+// accurate relative to itself (it is what the mean-field sum accumulates):
+//   2 (Q+ - Q-) = (G+ + G-)(dn+ - dn-) + (G+ - G-)(n+ + n-),
+//   a+ - a- = (dh+ - dh-) a+ a-,   T = a+ + a-,
+//   CS: G+ - G- = (a+ - a-) (T + T^2 - a+ a-)    PY: (a+ - a-) (3 T - 1)
+// (exact divided differences of the closures in a, which take four
+// operations fewer per pair than in s: 128^3 full shell, sigma 4, 0.543 ->
+// 0.517 ms).  One reciprocal of s+ s- for both ends, and G+ dn+ - G- dn- in place
+// of the products above, are cheaper still but less exact (u_z of the driven
+// 8 x 8 x 41 slit off by 3.3e-4 of max|u_x| instead of 1.1e-4): a product s- /
+// (s+ s-) has twice the error of a reciprocal, and next to a wall dn is as
+// large as n.
 // ---------------------------------------------------------------------------
 template <class T>
 __device__ __forceinline__ T fast_rcp(T x);
@@ -328,10 +334,17 @@ __device__ __forceinline__ float fast_rcp<float>(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// Newton-Raphson from the hardware's approximation r0 of 1/x (about 20 bits):
+// with e = 1 - x r0, 1/x = r0 (1 + e + e^2 + ...), cut after e^2 (e^3 ~ 2^-60).
+// Three FP64 operations where a rounded division takes about ten; the FP64 pipe
+// (two lanes per clock and SM) bounds the FP64 step.
 template <>
 __device__ __forceinline__ double fast_rcp<double>(double x)
 {
-    return 1.0 / x;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
 // a + b rounded as a sum: never contracted with a product into a multiply-add,
@@ -342,27 +355,26 @@ __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(
 template <int CL, class T>
 __device__ __forceinline__ void pair_weights(T s0, T noff, T dhp, T dnp, T dhm, T dnm, T &qp, T &qm, T &qd)
 {
-    const T np = noff + dnp, nm = noff + dnm;
     if (CL == 2) {
-        qp = T(2) * np;
-        qm = T(2) * nm;
+        qp = T(2) * (noff + dnp);
+        qm = T(2) * (noff + dnm);
         qd = T(4) * (dnp - dnm);
         return;
     }
-    const T sp = s0 - dhp, sm = s0 - dhm;
-    const T spm = sp * sm;
+    const T np = noff + dnp, nm = noff + dnm;
+    const T ap = fast_rcp<T>(s0 - dhp), am = fast_rcp<T>(s0 - dhm);
+    const T sum = add_rn(ap, am), prod = ap * am;
+    const T dif = (dhp - dhm) * prod;
     T gp, gm, gd;
     if (CL == 0) {
-        const T sp2 = sp * sp, sm2 = sm * sm;
-        const T rp = fast_rcp<T>(sp2 * sp), rm = fast_rcp<T>(sm2 * sm);
-        gp = fma(sp, rp, rp);
-        gm = fma(sm, rm, rm);
-        gd = (dhp - dhm) * (add_rn(sp2, sm2) + fma(spm, sp + sm, spm)) * (rp * rm);
+        const T ap2 = ap * ap, am2 = am * am;
+        gp = fma(ap2, ap, ap2);
+        gm = fma(am2, am, am2);
+        gd = dif * (fma(sum, sum, sum) - prod);
     } else {
-        const T rp = fast_rcp<T>(sp * sp), rm = fast_rcp<T>(sm * sm);
-        gp = fma(-sp, rp, T(3) * rp);
-        gm = fma(-sm, rm, T(3) * rm);
-        gd = (dhp - dhm) * fma(T(3), sp + sm, -spm) * (rp * rm);
+        gp = ap * fma(T(3), ap, T(-1));
+        gm = am * fma(T(3), am, T(-1));
+        gd = dif * fma(T(3), sum, T(-1));
     }
     qp = gp * np;
     qm = gm * nm;
@@ -392,26 +404,64 @@ struct ShellAcc {
     T t;
 };
 
-// Add the (+e, -e) pair with unit vector (kx, ky, kz) of +e.  khat(-e) = -khat(+e),
-// so W takes the sum of the two ends' Q (v' - v) and S the difference of
-// their Q v'.
+// What a (+e, -e) pair with unit vector (kx, ky, kz) of +e adds to the sums
+// before the products with khat.  khat(-e) = -khat(+e), so W takes the sum of
+// the two ends' Q (v' - v) and S the difference of their Q v'.
 template <class T>
-__device__ __forceinline__ void accumulate_pair(ShellAcc<T> &a, T kx, T ky, T kz, T qp, T qm, T qd, T vpx, T vpy,
-                                                T vpz, T vmx, T vmy, T vmz, T vx, T vy, T vz)
+struct PairTerms {
+    T dx, dy, dz, ks, qd, tq;
+};
+
+template <class T>
+__device__ __forceinline__ PairTerms<T> pair_terms(T kx, T ky, T kz, T qp, T qm, T qd, T vpx, T vpy, T vpz, T vmx,
+                                                   T vmy, T vmz, T vx, T vy, T vz)
 {
+    PairTerms<T> r;
     const T px = qp * vpx, py = qp * vpy, pz = qp * vpz;
-    const T dx = fma(-qm, vmx, px), dy = fma(-qm, vmy, py), dz = fma(-qm, vmz, pz);
+    r.dx = fma(-qm, vmx, px);
+    r.dy = fma(-qm, vmy, py);
+    r.dz = fma(-qm, vmz, pz);
     const T ex = fma(qm, vmx, px), ey = fma(qm, vmy, py), ez = fma(qm, vmz, pz);
-    const T tq = add_rn(qp, qm);
-    a.t += tq;
-    const T sx = fma(-tq, vx, ex), sy = fma(-tq, vy, ey), sz = fma(-tq, vz, ez);
-    a.Vx = fma(kx, qd, a.Vx); a.Vy = fma(ky, qd, a.Vy); a.Vz = fma(kz, qd, a.Vz);
-    const T ks = fma(kx, sx, fma(ky, sy, kz * sz));
-    a.Wx = fma(kx, ks, a.Wx); a.Wy = fma(ky, ks, a.Wy); a.Wz = fma(kz, ks, a.Wz);
-    a.Sxx = fma(kx, dx, a.Sxx); a.Syy = fma(ky, dy, a.Syy); a.Szz = fma(kz, dz, a.Szz);
-    a.Sxy = fma(ky, dx, fma(kx, dy, a.Sxy));
-    a.Sxz = fma(kz, dx, fma(kx, dz, a.Sxz));
-    a.Syz = fma(kz, dy, fma(ky, dz, a.Syz));
+    r.tq = add_rn(qp, qm);
+    const T sx = fma(-r.tq, vx, ex), sy = fma(-r.tq, vy, ey), sz = fma(-r.tq, vz, ez);
+    r.ks = fma(kx, sx, fma(ky, sy, kz * sz));
+    r.qd = qd;
+    return r;
+}
+
+template <class T>
+__device__ __forceinline__ void accumulate_terms(ShellAcc<T> &a, T kx, T ky, T kz, const PairTerms<T> &r)
+{
+    a.t += r.tq;
+    a.Vx = fma(kx, r.qd, a.Vx); a.Vy = fma(ky, r.qd, a.Vy); a.Vz = fma(kz, r.qd, a.Vz);
+    a.Wx = fma(kx, r.ks, a.Wx); a.Wy = fma(ky, r.ks, a.Wy); a.Wz = fma(kz, r.ks, a.Wz);
+    a.Sxx = fma(kx, r.dx, a.Sxx); a.Syy = fma(ky, r.dy, a.Syy); a.Szz = fma(kz, r.dz, a.Szz);
+    a.Sxy = fma(ky, r.dx, fma(kx, r.dy, a.Sxy));
+    a.Sxz = fma(kz, r.dx, fma(kx, r.dz, a.Sxz));
+    a.Syz = fma(kz, r.dy, fma(ky, r.dz, a.Syz));
+}
+
+// The pairs of (a, b, c), with unit vector (kx, ky, kz), and of (a, b, -c), with
+// (kx, ky, -kz): the sums and differences of their terms share the products
+// with khat (five operations fewer than two pairs).  In a state uniform in x
+// and y the two mean-field differences are each other's negatives bit for bit,
+// so V_x and V_y take an exact zero from every couple and keep no rounding of
+// V_z's size, a spurious force along the walls.
+template <class T>
+__device__ __forceinline__ void accumulate_couple(ShellAcc<T> &a, T kx, T ky, T kz, const PairTerms<T> &r,
+                                                  const PairTerms<T> &q)
+{
+    a.t += add_rn(r.tq, q.tq);
+    const T vs = add_rn(r.qd, q.qd), vd = add_rn(r.qd, -q.qd);
+    a.Vx = fma(kx, vs, a.Vx); a.Vy = fma(ky, vs, a.Vy); a.Vz = fma(kz, vd, a.Vz);
+    const T ws = r.ks + q.ks, wd = r.ks - q.ks;
+    a.Wx = fma(kx, ws, a.Wx); a.Wy = fma(ky, ws, a.Wy); a.Wz = fma(kz, wd, a.Wz);
+    const T xs = r.dx + q.dx, ys = r.dy + q.dy, zs = r.dz + q.dz;
+    const T xd = r.dx - q.dx, yd = r.dy - q.dy, zd = r.dz - q.dz;
+    a.Sxx = fma(kx, xs, a.Sxx); a.Syy = fma(ky, ys, a.Syy); a.Szz = fma(kz, zd, a.Szz);
+    a.Sxy = fma(ky, xs, fma(kx, ys, a.Sxy));
+    a.Sxz = fma(kz, xd, fma(kx, zs, a.Sxz));
+    a.Syz = fma(kz, yd, fma(ky, zs, a.Syz));
 }
 
 // Fields of one node from its shell sums: C = n (F^mf + F^viscous) with
@@ -756,7 +806,7 @@ __device__ __forceinline__ void shell_sums_generic(const KParams &p, const V4<T>
             hbv = hb[j];
         }
     };
-    for (int m = 0; m + 1 < p.nshell; m += 2) {     // (+e, -e) pairs
+    const auto terms = [&](int m) {                 // the (+e, -e) pair of entries m, m + 1
         const int4 e = shell_e[m];
         const V4<T> k = shell_k[m];
         V4<T> nb[2];
@@ -770,8 +820,17 @@ __device__ __forceinline__ void shell_sums_generic(const KParams &p, const V4<T>
             qm *= k.w;
             qd *= k.w;
         }
-        accumulate_pair<T>(a, k.x, k.y, k.z, qp, qm, qd, nb[0].y, nb[0].z, nb[0].w, nb[1].y, nb[1].z, nb[1].w, vx,
-                           vy, vz);
+        return pair_terms<T>(k.x, k.y, k.z, qp, qm, qd, nb[0].y, nb[0].z, nb[0].w, nb[1].y, nb[1].z, nb[1].w, vx, vy,
+                             vz);
+    };
+    const int nc = WT ? 0 : 4 * p.ncouple;
+    for (int m = 0; m < nc; m += 4) {               // mirror couples, as in the tiled kernel
+        const V4<T> k = shell_k[m];
+        accumulate_couple<T>(a, k.x, k.y, k.z, terms(m), terms(m + 2));
+    }
+    for (int m = nc; m + 1 < p.nshell; m += 2) {
+        const V4<T> k = shell_k[m];
+        accumulate_terms<T>(a, k.x, k.y, k.z, terms(m));
     }
 }
 
@@ -818,8 +877,8 @@ __device__ __forceinline__ void shell_body(const KParams &p, const KBufs<S, type
 
 // ---------------------------------------------------------------------------
 // Split form of shell_body: a block of kSplit warps serves 32 nodes, lane l of
-// every warp the same node, and warp k sums the pairs k, k + kSplit, ... of the
-// table; warp 0 adds the partial sums in warp order and runs the collision.
+// every warp the same node, and warp k sums the couples (then the pairs left
+// over) k, k + kSplit, ... of the table; warp 0 adds the partial sums in warp order and runs the collision.
 // Unsplit, the kernel is bound by each warp's own chain of loads and sums (FP32:
 // 381 pairs at sigma 8, ~400 instructions each) or by the FP64 pipe of the few
 // SMs that hold a block (two lanes a clock), so a lattice of few blocks leaves
@@ -831,7 +890,7 @@ __device__ __forceinline__ void shell_body(const KParams &p, const KBufs<S, type
 // sigma 8 on 8 x 8 x 256 (FP32) 256.8 -> 39.5 us, the 8 x 8 x 41 slit in FP64
 // 547 -> 94 us, a 48^3 box in FP64 1 697 -> 1 531 us (bound by the FP64 pipe).
 // ---------------------------------------------------------------------------
-constexpr int kSplit = 4;
+constexpr int kSplit = 4;   // eight warps: 96^3 at sigma 8 1 607 -> 2 149 us, FP64 45 x 38 x 51 1 055 -> 1 369
 
 template <class S, int CL, bool WALLS, bool WT, class A = typename Store<S>::T>
 __device__ __forceinline__ void shell_split_body(const KParams &p, const KBufs<S, typename Store<S>::T> &b, int node0)
@@ -859,16 +918,14 @@ __device__ __forceinline__ void shell_split_body(const KParams &p, const KBufs<S
     ShellAcc<T> a = {};
     if (fluid && p.interactions) {
         const T s0 = T(1) - hr - hoff;
-        const int npair = p.nshell >> 1;
-#pragma unroll 2
-        for (int m = wid; m < npair; m += kSplit) {
-            const int4 e = b.shell_e[2 * m];
-            const V4<T> k = b.shell_k[2 * m];
+        const auto terms = [&](int m) {             // the (+e, -e) pair of entries m, m + 1
+            const int4 e = b.shell_e[m];
+            const V4<T> k = b.shell_k[m];
             const int jp = axis[0][R + e.x][lane] + axis[1][R + e.y][lane] + axis[2][R + e.z][lane];
             const int jm = axis[0][R - e.x][lane] + axis[1][R - e.y][lane] + axis[2][R - e.z][lane];
-            if (!in_bounds(jp, p.N, b.status) || !in_bounds(jm, p.N, b.status)) continue;
-            const V4<T> np = b.nu[jp], nm = b.nu[jm];
-            const T hp = b.hb[jp], hm = b.hb[jm];
+            const bool ok = in_bounds(jp, p.N, b.status) && in_bounds(jm, p.N, b.status);
+            const V4<T> np = b.nu[ok ? jp : i], nm = b.nu[ok ? jm : i];
+            const T hp = b.hb[ok ? jp : i], hm = b.hb[ok ? jm : i];
             T qp, qm, qd;
             pair_weights<CL, T>(s0, noff, hp, np.x, hm, nm.x, qp, qm, qd);
             if (WT) {
@@ -876,7 +933,18 @@ __device__ __forceinline__ void shell_split_body(const KParams &p, const KBufs<S
                 qm *= k.w;
                 qd *= k.w;
             }
-            accumulate_pair<T>(a, k.x, k.y, k.z, qp, qm, qd, np.y, np.z, np.w, nm.y, nm.z, nm.w, me.y, me.z, me.w);
+            return pair_terms<T>(k.x, k.y, k.z, qp, qm, qd, np.y, np.z, np.w, nm.y, nm.z, nm.w, me.y, me.z, me.w);
+        };
+        const int nc = WT ? 0 : 4 * p.ncouple;
+#pragma unroll 2
+        for (int m = 4 * wid; m < nc; m += 4 * kSplit) {      // mirror couples, as in the tiled kernel
+            const V4<T> k = b.shell_k[m];
+            accumulate_couple<T>(a, k.x, k.y, k.z, terms(m), terms(m + 2));
+        }
+#pragma unroll 2
+        for (int m = nc + 2 * wid; m < p.nshell; m += 2 * kSplit) {
+            const V4<T> k = b.shell_k[m];
+            accumulate_terms<T>(a, k.x, k.y, k.z, terms(m));
         }
     }
     T *acc = reinterpret_cast<T *>(&a);

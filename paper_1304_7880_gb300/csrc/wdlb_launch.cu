@@ -74,8 +74,14 @@ void launch_fields_shell(const KParams &p, const KBufs<S, T> &b, cudaStream_t st
 template <int S2, int V, bool WALLS, bool WT>
 cudaError_t tiled_attr()
 {
-    return cudaFuncSetAttribute(k_step_shell_tiled<S, S2, V, WALLS, WT, A>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tiled::smem_bytes<S2, V, WT>());
+    const int smem = (int)tiled::smem_bytes<S2, V>();
+    cudaError_t e = cudaFuncSetAttribute(k_step_shell_tiled<S, S2, V, WALLS, WT, A>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if constexpr (!WT)
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_step_shell_tiled<S, S2, V, WALLS, WT, A, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return e;
 }
 
 template <int S2, int V, bool WT>
@@ -103,8 +109,14 @@ cudaError_t tiled_attr_r(int v, bool walls, bool wt)
 template <int S2, int V, bool WALLS, bool WT>
 void launch_tiled_group(const BatchLaunch &L, const KBufs<S, float> *B, const BatchGroup &G, cudaStream_t st)
 {
+    if constexpr (!WT)
+        if (G.roomy) {
+            k_step_shell_tiled<S, S2, V, WALLS, WT, A, true>
+                <<<G.nitems, tiled::threads_of(V), tiled::smem_bytes<S2, V>(), st>>>(L.params, B, G.items);
+            return;
+        }
     k_step_shell_tiled<S, S2, V, WALLS, WT, A>
-        <<<G.nitems, tiled::threads_of(V), tiled::smem_bytes<S2, V, WT>(), st>>>(L.params, B, G.items);
+        <<<G.nitems, tiled::threads_of(V), tiled::smem_bytes<S2, V>(), st>>>(L.params, B, G.items);
 }
 
 template <int S2, int V, bool WT>
@@ -144,26 +156,30 @@ void launch_tiled_v(const BatchLaunch &L, const KBufs<S, float> *B, const BatchG
 template <int S2, bool WT>
 bool compiled_table_matches()
 {
-    if constexpr (!tiled::ct::compiled<S2, WT>()) {
-        return true;
-    } else {
-        const double sigma = 0.5 * S2;
-        std::vector<int> e;
+    const double sigma = 0.5 * S2;
+    std::vector<int> e;
+    if constexpr (WT) {
         std::vector<double> wts;
-        double w = 0.0;
-        if (WT) {
-            if (!build_shell_compact(sigma, e, wts)) return false;
-        } else {
-            build_shell(sigma, e, &w);
-        }
+        if (!build_shell_compact(sigma, e, wts)) return false;
         constexpr tiled::ct::PairTable<S2, WT> T{};
         if ((int)e.size() != 6 * T.n) return false;
         for (int m = 0; m < T.n; m++) {
             if (e[6 * m] != T.ex[m] || e[6 * m + 1] != T.ey[m] || e[6 * m + 2] != T.ez[m]) return false;
-            if (WT && wts[2 * m] != wts[2 * tiled::ct::first_pair_of_orbit<S2>(T.orb[m])]) return false;
+            if (wts[2 * m] != wts[2 * tiled::ct::first_pair_of_orbit<S2>(T.orb[m])]) return false;
         }
-        return true;
+    } else {
+        double w = 0.0;
+        build_shell(sigma, e, &w);
+        const tiled::ct::FullTable<S2> &T = tiled::ct::kFull<S2>;
+        if (order_couples(e) != T.nc || (int)e.size() != 6 * (2 * T.nc + T.ns)) return false;
+        constexpr int SX = tiled::TX + 2 * tiled::shell_radius(S2);
+        for (int m = 0; m < 2 * T.nc + T.ns; m++) {
+            const tiled::ct::PairEntry &t = T.e[m < 2 * T.nc ? m / 2 : m - T.nc];
+            const int off = e[6 * m] + SX * (e[6 * m + 1] + SX * e[6 * m + 2]);
+            if ((m < 2 * T.nc && m % 2 ? t.q4 : t.p4) != 4 * off) return false;
+        }
     }
+    return true;
 }
 
 template <int S2>
@@ -366,7 +382,7 @@ template <bool WALLS, bool WT>
 cudaError_t launch_flow(const BatchLaunch &L, const FlowLaunch &F, cudaStream_t st)
 {
     auto kern = k_step_flow<S, 8, 2, WALLS, WT, A>;
-    const size_t smem = flow_smem_bytes<8, 2, WT>();
+    const size_t smem = flow_smem_bytes<8, 2>();
     static int grid = 0;   // one per template instance: resident blocks on the whole GPU
     if (grid == 0) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

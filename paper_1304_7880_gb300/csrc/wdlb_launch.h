@@ -42,6 +42,7 @@ struct BatchItem {
 struct BatchGroup {
     int s2, walls, tiled, closure, tile, rule;   // rule: shell rule (0 full, 1 compact)
     int split;                                   // generic kernel: pairs split over four warps
+    int roomy;                                   // tiled full shell: the form for launches of at most one block per SM
     const BatchItem *items;
     int nitems;
 };

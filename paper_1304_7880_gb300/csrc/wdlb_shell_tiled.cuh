@@ -16,13 +16,16 @@
 // The tile arrives by cp.async (16 bytes of nu, 4 of hb per node), so all
 // of a thread's halo loads are in flight together (measured 3 % faster for
 // the full sigma-4 shell, 8 to 18 % for the compact shells).
-// The (+e, -e) pairs of the contact shell are staged once per block as
-// (khat_x, khat_y, khat_z, offset of +e in the tile); the loop over them is
-// kept rolled (a few pairs per iteration) so the code stays in the
-// instruction cache.  Each pair goes through pair_weights and accumulate_pair,
-// the same arithmetic as shell_body.  WT (the compact shell): the pairs are
-// the first nshell/2 of the table, staged with their weights, which scale
-// each pair's Q as in shell_body.
+// The (+e, -e) pairs of the full shell sit in constant memory with their tile
+// offsets (ct::FullTable); the loop over them is kept rolled (two couples per
+// iteration) so the code stays in the instruction cache.  The kernel is bound by
+// instruction issue: a staged table and offsets cost 68 instructions per pair,
+// this form 60; with pair_weights' closed form and the couples the 128^3 box's
+// full shell took 0.543 -> 0.478 ms (sigma 4, FP32), the 96^3 box's at sigma 6
+// (FP16) 0.551 -> 0.474 ms.  Each pair goes through pair_weights, pair_terms and
+// accumulate_couple, the same arithmetic in the same order as shell_body.  WT
+// (the compact shell): the pairs are compiled in, with one weight per orbit that
+// scales each pair's Q as in shell_body.
 #pragma once
 
 #include <type_traits>
@@ -151,6 +154,63 @@ constexpr int first_pair_of_orbit(int o)
     return 0;
 }
 
+// Full shells: the pairs in constant memory, read at an index that is uniform
+// over the block, as couples (a, b, c), (a, b, -c) and the pairs left over
+// (c = 0 and a = b = 0): unit vector and, for the nu tile (16 bytes per node)
+// and the hb tile (4), the byte offsets of (a, b, c) and of (a, b, -c); a
+// single's second pair of offsets is unused.
+struct PairEntry {
+    float kx, ky, kz;
+    int p16, p4, m16, m4;         // +(a, b, c), -(a, b, c)
+    int q16, q4, r16, r4, pad;    // +(a, b, -c), -(a, b, -c)
+};
+
+template <int S2>
+struct FullTable {
+    int nc, ns;                   // couples, then singles from e[nc] on
+    PairEntry e[256];
+    constexpr FullTable() : nc(0), ns(0), e{}
+    {
+        const int R = (S2 + 1) / 2, SX = 8 + 2 * R;
+        int m = 0;
+        for (int pass = 0; pass < 2; pass++)
+            for (int dx = 0; dx <= R; dx++)
+                for (int dy = -R; dy <= R; dy++)
+                    for (int dz = 0; dz <= R; dz++) {
+                        const bool axis = dx == 0 && dy == 0;
+                        const bool positive = dx > 0 || dy > 0 || (axis && dz > 0);
+                        const int r2 = dx * dx + dy * dy + dz * dz;
+                        if ((dx == 0 && dy < 0) || !positive || !((S2 - 1) * (S2 - 1) < 4 * r2 && 4 * r2 <= (S2 + 1) * (S2 + 1)))
+                            continue;
+                        const bool couple = dz > 0 && !axis;
+                        if (couple != (pass == 0)) continue;
+                        const double len = sqrt_newton(double(r2));
+                        const int o = dx + SX * (dy + SX * dz), o2 = dx + SX * (dy - SX * dz);
+                        PairEntry &t = e[m++];
+                        t.kx = float(dx / len);
+                        t.ky = float(dy / len);
+                        t.kz = float(dz / len);
+                        t.p16 = 16 * o;
+                        t.p4 = 4 * o;
+                        t.m16 = -16 * o;
+                        t.m4 = -4 * o;
+                        t.q16 = 16 * o2;
+                        t.q4 = 4 * o2;
+                        t.r16 = -16 * o2;
+                        t.r4 = -4 * o2;
+                        if (couple)
+                            nc++;
+                        else
+                            ns++;
+                    }
+    }
+};
+
+template <int S2>
+constexpr FullTable<S2> kFull = FullTable<S2>();
+template <int S2>
+__constant__ FullTable<S2> c_full = FullTable<S2>();
+
 // Shells with a compiled table: the compact rule at sigma 3, 4 and 6 (13, 21
 // and 15 pairs; 7-10 % faster than the runtime table on the 128^3 box).  The
 // full shells keep the runtime loop: unrolled, their 49 to 225 pairs ran 4 %
@@ -215,13 +275,12 @@ __device__ __forceinline__ void accumulate_pair_ct(ShellAcc<float> &a, float qp,
 
 }  // namespace ct
 
-template <int S2, int V, bool WT = false>
+template <int S2, int V>
 constexpr size_t smem_bytes()
 {
     constexpr int R = shell_radius(S2);
     constexpr size_t n = size_t(TX + 2 * R) * (TY + 2 * R) * (tz_of(V) + 2 * R);
-    const size_t tables = size_t(shell_count(S2) / 2) * (sizeof(float4) + (WT ? sizeof(float) : 0));
-    return n * (sizeof(float4) + sizeof(float)) + (tables + 7) / 8 * 8 + sizeof(uint64_t);   // + the mbarrier
+    return n * (sizeof(float4) + sizeof(float)) + sizeof(uint64_t);   // + the mbarrier
 }
 
 // TMA staging of the tile: for a halo R that is a multiple of 4 (sigma 4),
@@ -240,16 +299,22 @@ constexpr bool tma_staging()
 // threads.  Three blocks measured 7-12 % faster than two for sigma 3 (8^3
 // bricks) and sigma 4 (8 x 8 x 4 bricks), and 5 % faster for the double-word
 // collision at sigma 4, whose 85 registers spill ~100 bytes.
-template <int S2, int V, bool WT = false>
+// ROOMY: one block, for launches of at most one block per SM, where a second
+// has nothing to run; the registers go into four couples per iteration, whose
+// loads and reciprocals overlap (8 x 8 x 41 slit, sigma 4: 50 steps 1.16 -> 1.09
+// ms; 27 x 27 x 46, sigma 3, 96 bricks: 100 steps 2.55 -> 2.38 ms; on 128^3
+// 0.474 -> 0.481 ms).  The sums are the same bits.
+template <int S2, int V, bool ROOMY = false>
 constexpr int blocks_per_sm()
 {
-    return threads_of(V) != 256                                ? 1
-           : 3 * smem_bytes<S2, V, WT>() <= size_t(227) * 1024 ? 3
-           : 2 * smem_bytes<S2, V, WT>() <= size_t(227) * 1024 ? 2
+    return ROOMY || threads_of(V) != 256                       ? 1
+           : 3 * smem_bytes<S2, V>() <= size_t(227) * 1024 ? 3
+           : 2 * smem_bytes<S2, V>() <= size_t(227) * 1024 ? 2
                                                                 : 1;
 }
 
-template <class S, int S2, int V, int CL, bool WALLS, bool FIELDS, bool WT = false, class A = float>
+template <class S, int S2, int V, int CL, bool WALLS, bool FIELDS, bool WT = false, class A = float,
+          bool ROOMY = false>
 __device__ __forceinline__ void tiled_body(const KParams &p, const KBufs<S, float> &b, int bx, int by, int bz)
 {
     constexpr int R = shell_radius(S2);
@@ -264,26 +329,14 @@ __device__ __forceinline__ void tiled_body(const KParams &p, const KBufs<S, floa
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float4 *sm4 = reinterpret_cast<float4 *>(smem_raw);
     float *smh = reinterpret_cast<float *>(smem_raw + sizeof(float4) * NS);
-    float4 *smt = reinterpret_cast<float4 *>(smem_raw + (sizeof(float4) + sizeof(float)) * NS);
-    float *smw = reinterpret_cast<float *>(smt + NPAIR);   // pair weights (WT)
     uint64_t *bar = reinterpret_cast<uint64_t *>(
-        smem_raw + smem_bytes<S2, V, WT>() - sizeof(uint64_t));
-    static_assert(((sizeof(float4) + sizeof(float)) * NS) % 16 == 0, "pair table alignment");
-    const int npair = WT ? (p.nshell >> 1) : NPAIR;
+        smem_raw + smem_bytes<S2, V>() - sizeof(uint64_t));
+    static_assert(((sizeof(float4) + sizeof(float)) * NS) % 8 == 0, "mbarrier alignment");
     constexpr bool CT = ct::compiled<S2, WT>();
 
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const int x0 = bx * TX, y0 = by * TY, z0 = bz * TZ;
 
-    // shell pairs: +e is entry 2m of the library's table (-e is 2m + 1)
-    if constexpr (!CT) {
-        for (int m = threadIdx.x; m < npair; m += NT) {
-            const int4 e = b.shell_e[2 * m];
-            const V4<float> k = b.shell_k[2 * m];
-            smt[m] = make_float4(k.x, k.y, k.z, __int_as_float(e.x + SX * (e.y + SY * e.z)));
-            if (WT) smw[m] = k.w;
-        }
-    }
     // compiled table with the compact rule: the weight of each orbit, taken
     // from the first pair of the orbit in the library's table
     float wo[3] = {1.f, 1.f, 1.f};
@@ -403,27 +456,44 @@ __device__ __forceinline__ void tiled_body(const KParams &p, const KBufs<S, floa
                                                        me.z, me.w);
                 });
             }
-            // three pairs per iteration; kept rolled for sigma 6 (225 pairs), where
-            // it measured 1.5 % faster
-#pragma unroll(S2 >= 12 && !WT ? 1 : 3)
-            for (int m = 0; m < (CT ? 0 : npair); m++) {
-                const float4 t = smt[m];
-                const int off = __float_as_int(t.w);
-                if (!in_bounds(base + off, NS, b.status) || !in_bounds(base - off, NS, b.status)) continue;
-                const float4 np = sm4[base + off];
-                const float hp = smh[base + off];
-                const float4 nm = sm4[base - off];
-                const float hm = smh[base - off];
-                float qp, qm, qd;
-                pair_weights<CL, float>(s0, noff, hp, np.x, hm, nm.x, qp, qm, qd);
-                if (WT) {
-                    const float r = smw[m];
-                    qp *= r;
-                    qm *= r;
-                    qd *= r;
-                }
-                accumulate_pair<float>(a, t.x, t.y, t.z, qp, qm, qd, np.y, np.z, np.w, nm.y, nm.z, nm.w, me.y,
-                                       me.z, me.w);
+            // The runtime loop over the full shell: 60 instructions per pair (54
+            // multiply-adds, two reciprocals, four loads).  Table and offsets
+            // come through uniform registers, so an address takes none; two
+            // couples per iteration for sigma 3 and 4 (1, 3 and 4 measured 3, 1
+            // and 1.5 % slower), one for sigma 6.
+            constexpr int kUnroll = ROOMY ? 4 : S2 >= 12 ? 1 : 2;
+            if constexpr (!CT) {
+                constexpr int NC = ct::kFull<S2>.nc, NSI = ct::kFull<S2>.ns;
+                static_assert(2 * NC + NSI == NPAIR, "couples and singles cover the shell");
+                const char *c16 = reinterpret_cast<const char *>(sm4 + base);
+                const char *c4 = reinterpret_cast<const char *>(smh + base);
+                const auto inside = [&](int o4) { return in_bounds(base + o4 / 4, NS, b.status); };
+                const auto terms = [&](int p16, int p4, int m16, int m4, float kx, float ky, float kz) {
+                    const float4 np = *reinterpret_cast<const float4 *>(c16 + p16);
+                    const float hp = *reinterpret_cast<const float *>(c4 + p4);
+                    const float4 nm = *reinterpret_cast<const float4 *>(c16 + m16);
+                    const float hm = *reinterpret_cast<const float *>(c4 + m4);
+                    float qp, qm, qd;
+                    pair_weights<CL, float>(s0, noff, hp, np.x, hm, nm.x, qp, qm, qd);
+                    return pair_terms<float>(kx, ky, kz, qp, qm, qd, np.y, np.z, np.w, nm.y, nm.z, nm.w, me.y, me.z,
+                                             me.w);
+                };
+                const auto couple = [&](int m) {
+                    const ct::PairEntry &t = ct::c_full<S2>.e[m];
+                    if (!inside(t.p4) || !inside(t.m4) || !inside(t.q4) || !inside(t.r4)) return;
+                    accumulate_couple<float>(a, t.kx, t.ky, t.kz, terms(t.p16, t.p4, t.m16, t.m4, t.kx, t.ky, t.kz),
+                                             terms(t.q16, t.q4, t.r16, t.r4, t.kx, t.ky, -t.kz));
+                };
+                const auto single = [&](int m) {
+                    const ct::PairEntry &t = ct::c_full<S2>.e[m];
+                    if (!inside(t.p4) || !inside(t.m4)) return;
+                    accumulate_terms<float>(a, t.kx, t.ky, t.kz,
+                                            terms(t.p16, t.p4, t.m16, t.m4, t.kx, t.ky, t.kz));
+                };
+#pragma unroll kUnroll
+                for (int m = 0; m < NC; m++) couple(m);
+#pragma unroll kUnroll
+                for (int m = NC; m < NC + NSI; m++) single(m);
             }
             shell_forces<float>(p, a, noff + me.x, me.y, me.z, me.w, Cx, Cy, Cz, Axx, Ayy, Azz, Axy, Axz, Ayz,
                                 tsum);

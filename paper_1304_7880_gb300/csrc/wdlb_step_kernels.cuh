@@ -74,14 +74,14 @@ __global__ void __launch_bounds__(32 * kSplit)
     shell_split_body<S, CL, WALLS, WT, A>(p, b, node0);
 }
 
-template <class S, int S2, int V, bool WALLS, bool WT, class A = float>
-__global__ void __launch_bounds__(tiled::threads_of(V), (tiled::blocks_per_sm<S2, V, WT>()))
+template <class S, int S2, int V, bool WALLS, bool WT, class A = float, bool ROOMY = false>
+__global__ void __launch_bounds__(tiled::threads_of(V), (tiled::blocks_per_sm<S2, V, ROOMY>()))
     k_step_shell_tiled(const KParams *P, const KBufs<S, float> *B, const BatchItem *it)
 {
     const BatchItem w = it[blockIdx.x];
     const KParams p = P[w.slot];
     const KBufs<S, float> b = B[w.slot];
-    tiled::tiled_body<S, S2, V, 0, WALLS, false, WT, A>(p, b, w.bx, w.by, w.bz);
+    tiled::tiled_body<S, S2, V, 0, WALLS, false, WT, A, ROOMY>(p, b, w.bx, w.by, w.bz);
 }
 
 }  // namespace wdlb
@@ -122,10 +122,10 @@ struct FlowArgs {
 
 // dynamic shared memory of the flow kernel: the shell tile (the largest of the
 // three phases) and 16 bytes for the block's item and stop flag
-template <int S2, int V, bool WT>
+template <int S2, int V>
 constexpr size_t flow_smem_bytes()
 {
-    return tiled::smem_bytes<S2, V, WT>() + 16;
+    return tiled::smem_bytes<S2, V>() + 16;
 }
 
 __device__ __forceinline__ int ld_acquire_gpu(const int *p)
@@ -136,7 +136,7 @@ __device__ __forceinline__ int ld_acquire_gpu(const int *p)
 }
 
 template <class S, int S2, int V, bool WALLS, bool WT, class A = float>
-__global__ void __launch_bounds__(tiled::threads_of(V), (tiled::blocks_per_sm<S2, V, WT>()))
+__global__ void __launch_bounds__(tiled::threads_of(V), (tiled::blocks_per_sm<S2, V>()))
     k_step_flow(FlowArgs a)
 {
     typedef typename Store<S>::T T;
@@ -144,8 +144,8 @@ __global__ void __launch_bounds__(tiled::threads_of(V), (tiled::blocks_per_sm<S2
     // the block's item and stop flag, past the shell tile in dynamic shared
     // memory (static shared memory would move the tile off its alignment)
     extern __shared__ __align__(128) unsigned char flow_smem[];
-    int &s_item = reinterpret_cast<int *>(flow_smem + flow_smem_bytes<S2, V, WT>() - 16)[0];
-    int &s_stop = reinterpret_cast<int *>(flow_smem + flow_smem_bytes<S2, V, WT>() - 16)[1];
+    int &s_item = reinterpret_cast<int *>(flow_smem + flow_smem_bytes<S2, V>() - 16)[0];
+    int &s_stop = reinterpret_cast<int *>(flow_smem + flow_smem_bytes<S2, V>() - 16)[1];
     const long long per_step = (long long)a.n0 + a.n1 + a.n2;
     const long long total = per_step * a.nsteps;
     const bool probe = a.wait_limit < 0;

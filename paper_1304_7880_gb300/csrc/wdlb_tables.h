@@ -53,6 +53,33 @@ inline void build_shell(double sigma, std::vector<int> &out, double *w)
     *w = second > 0 ? (4.0 * M_PI / 3.0) * sigma / second : 0.0;
 }
 
+// Reorder a full shell for the kernels: first the couples, the pair of (a, b, c)
+// followed by that of (a, b, -c), c > 0 and (a, b) != (0, 0), then the pairs
+// left over; each part in the order of build_shell.  Returns the number of
+// couples.
+inline int order_couples(std::vector<int> &v)
+{
+    std::vector<int> out;
+    int nc = 0;
+    auto put = [&](int x, int y, int z) {
+        for (int c : {x, y, z, -x, -y, -z}) out.push_back(c);
+    };
+    for (int pass = 0; pass < 2; pass++)
+        for (size_t m = 0; m + 5 < v.size(); m += 6) {
+            const int x = v[m], y = v[m + 1], z = v[m + 2];
+            const bool axis = x == 0 && y == 0;
+            if (pass == 0 && z > 0 && !axis) {
+                put(x, y, z);
+                put(x, y, -z);
+                nc++;
+            } else if (pass == 1 && (z == 0 || axis)) {
+                put(x, y, z);
+            }
+        }
+    v.swap(out);
+    return nc;
+}
+
 // Compact contact shell (shell rule 1; a quadrature of this library, the
 // paper leaves the discrete integral over khat of Eq. campoc open): two or
 // three orbits of the cubic group inside the full shell, one weight per orbit,
