@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 namespace wdlb {
 
 constexpr int NQ = 19;
@@ -115,17 +117,27 @@ __device__ __forceinline__ float prm<float>(double, float f) { return f; }
 constexpr int kMaxShellR = 8;    // floor(sigma + 1/2) for sigma <= 8
 
 // Tiled ball sum: an 8 x 8 x 8 brick of nodes per block with a halo of
-// ball_r, the brick's n - n_off and the ball's offsets in shared memory.
+// ball_r, the brick's n - n_off and the ball's offsets (or the brick's
+// row indices, side^2) in shared memory.
 constexpr int kBallTile = 8;
+constexpr int kBallThreads = 256;
 
 // Output brick depth of tile variant v of the tiled shell kernel.
 inline __host__ __device__ int tile_depth(int v) { return v == 2 ? 4 : 8; }
 constexpr size_t kBallTileMaxSmem = 48 * 1024;   // no opt-in attribute needed
 
-inline __host__ __device__ size_t ball_tile_smem(int ball_r, int nball, size_t tsize)
+// Row pitch of the brick in shared memory: 24 values put the four rows of eight
+// that a warp reads into different banks; the bare side where 24 would not fit
+// (FP64 at ball_r 4).
+inline __host__ __device__ constexpr int ball_pitch(int side, size_t tsize)
+{
+    return side <= 24 && size_t(side) * side * (24 * tsize + sizeof(int)) <= kBallTileMaxSmem ? 24 : side;
+}
+
+inline size_t ball_tile_smem(int ball_r, int nball, size_t tsize)
 {
     const size_t side = size_t(kBallTile + 2 * ball_r);
-    return side * side * side * tsize + size_t(nball) * sizeof(int);
+    return side * side * ball_pitch((int)side, tsize) * tsize + std::max(size_t(nball), side * side) * sizeof(int);
 }
 
 // Device buffers of one lattice.  S: storage type of populations; T: compute type.

@@ -190,8 +190,7 @@ __device__ __forceinline__ void ball_body(const KParams &p, const V4<T> *nu, T *
     hb[i] = dh;
 }
 
-// Tiled form of ball_body: one 8 x 8 x 8 brick of nodes per block of 256
-// threads (two nodes per thread, z and z + 4), with n - n_off of the brick
+// Tiled form of ball_body: one 8 x 8 x 8 brick of nodes per block, with n - n_off of the brick
 // and its halo of ball_r, and the ball's offsets within it, in shared memory.
 // Beyond a wall the staged value is -n_off (n = 0).  The brick arrives by
 // cp.async (all of a thread's loads in flight at once).  The ball points are
@@ -227,9 +226,8 @@ __device__ __forceinline__ void ball_tiled_body(const KParams &p, const V4<T> *n
     }
     cp_async_wait_all();
     __syncthreads();
-    const int tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7, tzb = threadIdx.x >> 6;
-    for (int half = 0; half < 2; half++) {
-        const int tz = tzb + 4 * half;
+    const int tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7;
+    for (int tz = threadIdx.x >> 6; tz < kBallTile; tz += blockDim.x >> 6) {
         const int x = x0 + tx, y = y0 + ty, z = z0 + tz;
         if (x >= p.nx || y >= p.ny || z >= p.nz) continue;
         const int i = x + p.nx * (y + p.ny * z);
@@ -248,58 +246,97 @@ __device__ __forceinline__ void ball_tiled_body(const KParams &p, const V4<T> *n
 }
 
 // ball_tiled_body with 2 sigma = S2 known at compile time (sigma 3, 4, 6, 8): the
-// brick side and the ball's offsets are constants, and the points are added
-// in the order of the host's ball table (dx, then dy, then dz ascending), so
-// the sums are bitwise those of ball_body and ball_tiled_body.
-template <class T, int S2>
+// brick side and the ball's offsets are constants.  NT threads: each sums
+// ZO = 512/NT nodes of a z column, so that one load of a column's value serves
+// every output whose window it lies in (sigma 4, two outputs: 23 loads per
+// output for 33 points; sigma 6: 76 for 123).  A thread stages one x of every
+// RP-th row of the brick, from row indices formed once, and only as far beyond
+// the brick as the ball reaches in that row.  Bound by the shared-memory and L1
+// pipes (8 bytes per node of the 16 that nu moves are needed): smeared density
+// of 128^3 at sigma 4 36.4 -> 25.3 us, 96^3 at sigma 6 40.0 -> 20.4, 64 pores
+// 75 -> 48, a serving mix 100 -> 54.  128 threads: 27.6, 20.3, 54.7, 54.2.  A
+// dense copy of n - n_off for this kernel made it 21.4 us, and the moments, which
+// write the copy, 2 to 6 us slower.
+// Each output adds the ball's points in the order of the host's table (dx, then
+// dy, then dz ascending), so the sums are bitwise those of ball_body and
+// ball_tiled_body.
+template <class T, int S2, int NT>
 __device__ __forceinline__ void ball_brick_ct(const KParams &p, const V4<T> *nu, T *hb, int *status, int bx,
                                               int by, int bz)
 {
     constexpr int R = S2 / 4;                       // floor(sigma / 2)
-    constexpr int SX = kBallTile + 2 * R, NS = SX * SX * SX;
+    constexpr int SX = kBallTile + 2 * R, PX = ball_pitch(SX, sizeof(T)), NS = PX * SX * SX;
+    constexpr int ZO = kBallTile * kBallTile * kBallTile / NT;
     extern __shared__ __align__(16) unsigned char ball_smem[];
     T *sn = reinterpret_cast<T *>(ball_smem);
+    int *rows = reinterpret_cast<int *>(ball_smem + size_t(NS) * sizeof(T));   // [SX * SX]
     const T noff = prm<T>(p.n_off, p.f_n_off);
+    const int nx = p.nx, ny = p.ny, nz = p.nz;
     const int x0 = bx * kBallTile, y0 = by * kBallTile, z0 = bz * kBallTile;
-    for (int idx = threadIdx.x; idx < NS; idx += blockDim.x) {
-        const int sx = idx % SX, sy = (idx / SX) % SX, sz = idx / (SX * SX);
-        const int gx = wrap_coord(x0 - R + sx, p.nx), gy = wrap_coord(y0 - R + sy, p.ny);
-        int gz = z0 - R + sz;
-        bool inside = true;
-        if (p.walls)
-            inside = gz >= 0 && gz < p.nz;
-        else
-            gz = wrap_coord(gz, p.nz);
-        const int g = gx + p.nx * (gy + p.ny * gz);
-        if (inside && in_bounds(g, p.N, status))
-            cp_async_ca<sizeof(T)>(sn + idx, &nu[g].x);
-        else
-            sn[idx] = -noff;
+    // a row's first index and how far beyond the brick in x the ball reaches in
+    // it (-1: no ball point lies in the row), 8 index + reach + 1; beyond a wall
+    // the index is -1
+    for (int r = threadIdx.x; r < SX * SX; r += NT) {
+        const int sy = r % SX - R, sz = r / SX - R;
+        const int oy = max(0, max(-sy, sy - kBallTile + 1)), oz = max(0, max(-sz, sz - kBallTile + 1));
+        int reach = R;
+        while (reach >= 0 && 16 * (reach * reach + oy * oy + oz * oz) > S2 * S2) reach--;
+        const int gz = z0 + sz, gy = wrap_coord(y0 + sy, ny);
+        const int g = p.walls && !(gz >= 0 && gz < nz) ? -1 : nx * (gy + ny * wrap_coord(gz, nz));
+        rows[r] = 8 * g + reach + 1;
+    }
+    __syncthreads();
+    constexpr int RP = NT / SX;                     // rows a pass of the block stages
+    if (threadIdx.x < RP * SX) {
+        const int sx = threadIdx.x % SX;
+        const int gx = wrap_coord(x0 - R + sx, nx);
+        const int ox = max(0, max(R - sx, sx - R - kBallTile + 1));   // how far this x lies beyond the brick
+#pragma unroll 4
+        for (int r = threadIdx.x / SX; r < SX * SX; r += RP) {
+            const int e = rows[r];
+            if ((e & 7) <= ox) continue;
+            const int g = e >> 3;
+            if (g >= 0 && in_bounds(g + gx, p.N, status))
+                cp_async_ca<sizeof(T)>(sn + r * PX + sx, &nu[g + gx].x);
+            else
+                sn[r * PX + sx] = -noff;
+        }
     }
     cp_async_wait_all();
     __syncthreads();
-    const int tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7, tzb = threadIdx.x >> 6;
-    for (int half = 0; half < 2; half++) {
-        const int tz = tzb + 4 * half;
-        const int x = x0 + tx, y = y0 + ty, z = z0 + tz;
-        if (x >= p.nx || y >= p.ny || z >= p.nz) continue;
-        const int i = x + p.nx * (y + p.ny * z);
+    const int tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7, tz = (threadIdx.x >> 6) * ZO;
+    const int x = x0 + tx, y = y0 + ty;
+    if (x >= nx || y >= ny) return;
+    const T *c = sn + (tx + R) + PX * ((ty + R) + SX * (tz + R));
+    T sum[ZO] = {};
+#pragma unroll
+    for (int dx = -R; dx <= R; dx++)
+#pragma unroll
+        for (int dy = -R; dy <= R; dy++) {
+            T v[ZO + 2 * R];                        // the column's values at dz = -R .. R + ZO - 1
+#pragma unroll
+            for (int k = 0; k < ZO + 2 * R; k++) {
+                const int dz = k < R ? k - R : (k >= ZO + R ? k - R - ZO + 1 : 0);   // its smallest |dz|
+                if (16 * (dx * dx + dy * dy + dz * dz) <= S2 * S2 &&
+                    in_bounds(c - sn + dx + PX * (dy + SX * (k - R)), NS, status))
+                    v[k] = c[dx + PX * (dy + SX * (k - R))];
+            }
+#pragma unroll
+            for (int o = 0; o < ZO; o++)
+#pragma unroll
+                for (int dz = -R; dz <= R; dz++)
+                    if (16 * (dx * dx + dy * dy + dz * dz) <= S2 * S2) sum[o] += v[o + dz + R];
+        }
+#pragma unroll
+    for (int o = 0; o < ZO; o++) {
+        const int z = z0 + tz + o;
+        if (z >= nz) break;
+        const int i = x + nx * (y + ny * z);
         if (solid_plane(p, z)) {
             hb[i] = -prm<T>(p.h_off, p.f_h_off);
             continue;
         }
-        const T *c = sn + (tx + R) + SX * ((ty + R) + SX * (tz + R));
-        T sum = T(0);
-#pragma unroll
-        for (int dx = -R; dx <= R; dx++)
-#pragma unroll
-            for (int dy = -R; dy <= R; dy++)
-#pragma unroll
-                for (int dz = -R; dz <= R; dz++)
-                    if (16 * (dx * dx + dy * dy + dz * dz) <= S2 * S2 &&
-                        in_bounds(c - sn + dx + SX * (dy + SX * dz), NS, status))
-                        sum += c[dx + SX * (dy + SX * dz)];
-        T dh = prm<T>(p.c_half, p.f_c_half) * sum;
+        const T dh = prm<T>(p.c_half, p.f_c_half) * sum[o];
         if (!(prm<T>(p.h_off, p.f_h_off) + dh < T(0.5))) atomicOr(status, 1);
         hb[i] = dh;
     }

@@ -319,7 +319,7 @@ cudaError_t do_batch_step(const BatchLaunch &L, int parity, int part, int group,
     }
     if (part < 0 || part == 1) {
         if (L.n_ball_items > 0) {
-            k_step_ball_tiled<S><<<L.n_ball_items, kThreads, L.ball_smem, st>>>(L.params, B, L.ball_items);
+            k_step_ball_tiled<S><<<L.n_ball_items, kBallThreads, L.ball_smem, st>>>(L.params, B, L.ball_items);
             *launches += 1;
         }
         if (L.n_ball_node_items > 0) {

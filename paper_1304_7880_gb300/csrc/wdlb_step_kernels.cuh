@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(256) k_step_ball(const KParams *P, const KBufs
 }
 
 template <class S>
-__global__ void __launch_bounds__(256) k_step_ball_tiled(const KParams *P, const KBufs<S, typename Store<S>::T> *B,
+__global__ void __launch_bounds__(kBallThreads) k_step_ball_tiled(const KParams *P, const KBufs<S, typename Store<S>::T> *B,
                                                          const BatchItem *it)
 {
     const BatchItem w = it[blockIdx.x];
@@ -41,10 +41,10 @@ __global__ void __launch_bounds__(256) k_step_ball_tiled(const KParams *P, const
     const KBufs<S, typename Store<S>::T> b = B[w.slot];
     typedef typename Store<S>::T T;
     switch (p.s2) {      // uniform over the block (one slot per block)
-    case 6: ball_brick_ct<T, 6>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
-    case 8: ball_brick_ct<T, 8>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
-    case 12: ball_brick_ct<T, 12>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
-    case 16: ball_brick_ct<T, 16>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
+    case 6: ball_brick_ct<T, 6, kBallThreads>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
+    case 8: ball_brick_ct<T, 8, kBallThreads>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
+    case 12: ball_brick_ct<T, 12, kBallThreads>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
+    case 16: ball_brick_ct<T, 16, kBallThreads>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
     default: ball_tiled_body<T>(p, b.nu, b.hb, b.ball, b.status, w.bx, w.by, w.bz); break;
     }
 }
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(tiled::threads_of(V), (tiled::blocks_per_sm<S2
         if (phase == 0)
             moments_body<S, false>(p, b, w.bx, nullptr, nullptr);
         else if (phase == 1)
-            ball_brick_ct<T, S2>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz);
+            ball_brick_ct<T, S2, 256>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz);
         else
             tiled::tiled_body<S, S2, V, 0, WALLS, false, WT, A>(p, b, w.bx, w.by, w.bz);
         __syncthreads();       // every thread's writes of this item are done
