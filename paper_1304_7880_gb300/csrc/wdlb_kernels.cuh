@@ -901,9 +901,7 @@ __device__ __forceinline__ void shell_sums_generic(const KParams &p, const V4<T>
             hbv = hb[j];
         }
     };
-    const auto terms = [&](int m) {                 // the (+e, -e) pair of entries m, m + 1
-        const int4 e = shell_e[m];
-        const V4<T> k = shell_k[m];
+    const auto terms = [&](int4 e, V4<T> k) {       // the (+e, -e) pair with unit vector k of +e
         V4<T> nb[2];
         T hbv[2];
         fetch(e.x, e.y, e.z, nb[0], hbv[0]);
@@ -920,12 +918,14 @@ __device__ __forceinline__ void shell_sums_generic(const KParams &p, const V4<T>
     };
     const int nc = WT ? 0 : 4 * p.ncouple;
     for (int m = 0; m < nc; m += 4) {               // mirror couples, as in the tiled kernel
+        const int4 e = shell_e[m];
         const V4<T> k = shell_k[m];
-        accumulate_couple<T>(a, k.x, k.y, k.z, terms(m), terms(m + 2));
+        accumulate_couple<T>(a, k.x, k.y, k.z, terms(e, k),
+                             terms(make_int4(e.x, e.y, -e.z, 0), V4<T>{k.x, k.y, -k.z, k.w}));
     }
     for (int m = nc; m + 1 < p.nshell; m += 2) {
         const V4<T> k = shell_k[m];
-        accumulate_terms<T>(a, k.x, k.y, k.z, terms(m));
+        accumulate_terms<T>(a, k.x, k.y, k.z, terms(shell_e[m], k));
     }
 }
 
@@ -981,11 +981,15 @@ __device__ __forceinline__ void shell_body(const KParams &p, const KBufs<S, type
 // sums.  Wrapped neighbour coordinates are formed once per node and shell
 // component (2 R + 1 per axis) into shared memory; beyond a wall they point at
 // the solid plane z = 0, whose nu and hb hold the n = 0 state, so a neighbour's
-// index is the sum of three words with no test.  Shell kernel, before and now:
-// sigma 8 on 8 x 8 x 256 (FP32) 256.8 -> 39.5 us, the 8 x 8 x 41 slit in FP64
-// 547 -> 94 us, a 48^3 box in FP64 1 697 -> 1 531 us (bound by the FP64 pipe).
+// index is the sum of three words with no test.  A couple takes one table entry:
+// its second pair is the first with z negated (sigma 8 on 8 x 8 x 256 41.2 ->
+// 31.1 us, 96^3 1 602 -> 1 238).  Shell kernel, unsplit with modulo wraps and now:
+// sigma 8 on 8 x 8 x 256 (FP32) 256.8 -> 31.1 us, bound by the latency of its
+// dependent loads (3.4 warps per scheduler); the 8 x 8 x 41 slit in FP64 547 -> 74
+// us, a 45 x 38 x 51 box in FP64 1 633 -> 1 005, bound by the FP64 pipe (about 55
+// operations per pair, two lanes per clock and SM).
 // ---------------------------------------------------------------------------
-constexpr int kSplit = 4;   // eight warps: 96^3 at sigma 8 1 607 -> 2 149 us, FP64 45 x 38 x 51 1 055 -> 1 369
+constexpr int kSplit = 4;   // (eight: 96^3 at sigma 8 1 607 -> 2 149 us, FP64 45 x 38 x 51 1 055 -> 1 369)
 
 template <class S, int CL, bool WALLS, bool WT, class A = typename Store<S>::T>
 __device__ __forceinline__ void shell_split_body(const KParams &p, const KBufs<S, typename Store<S>::T> &b, int node0)
@@ -1013,9 +1017,7 @@ __device__ __forceinline__ void shell_split_body(const KParams &p, const KBufs<S
     ShellAcc<T> a = {};
     if (fluid && p.interactions) {
         const T s0 = T(1) - hr - hoff;
-        const auto terms = [&](int m) {             // the (+e, -e) pair of entries m, m + 1
-            const int4 e = b.shell_e[m];
-            const V4<T> k = b.shell_k[m];
+        const auto terms = [&](int4 e, V4<T> k) {   // the (+e, -e) pair with unit vector k of +e
             const int jp = axis[0][R + e.x][lane] + axis[1][R + e.y][lane] + axis[2][R + e.z][lane];
             const int jm = axis[0][R - e.x][lane] + axis[1][R - e.y][lane] + axis[2][R - e.z][lane];
             const bool ok = in_bounds(jp, p.N, b.status) && in_bounds(jm, p.N, b.status);
@@ -1033,13 +1035,15 @@ __device__ __forceinline__ void shell_split_body(const KParams &p, const KBufs<S
         const int nc = WT ? 0 : 4 * p.ncouple;
 #pragma unroll 2
         for (int m = 4 * wid; m < nc; m += 4 * kSplit) {      // mirror couples, as in the tiled kernel
+            const int4 e = b.shell_e[m];
             const V4<T> k = b.shell_k[m];
-            accumulate_couple<T>(a, k.x, k.y, k.z, terms(m), terms(m + 2));
+            accumulate_couple<T>(a, k.x, k.y, k.z, terms(e, k),
+                                 terms(make_int4(e.x, e.y, -e.z, 0), V4<T>{k.x, k.y, -k.z, k.w}));
         }
 #pragma unroll 2
         for (int m = nc + 2 * wid; m < p.nshell; m += 2 * kSplit) {
             const V4<T> k = b.shell_k[m];
-            accumulate_terms<T>(a, k.x, k.y, k.z, terms(m));
+            accumulate_terms<T>(a, k.x, k.y, k.z, terms(b.shell_e[m], k));
         }
     }
     T *acc = reinterpret_cast<T *>(&a);

@@ -295,8 +295,8 @@ constexpr bool tma_staging()
 
 // Blocks per SM the launch bounds ask for: for 256 threads, three where three
 // blocks' shared memory fits (227 KB per SM; the compiler then keeps to 85
-// registers per thread), else two where two fit, else one.  Three blocks measured 7-12 % faster than two for sigma 3 (8^3
-// bricks) and sigma 4 (8 x 8 x 4 bricks), and 5 % faster for the double-word
+// registers per thread), else two where two fit, else one.  Three blocks
+// measured 7-12 % faster than two for sigma 3 (8^3 bricks) and sigma 4 (8 x 8 x 4 bricks), and 5 % faster for the double-word
 // collision at sigma 4, whose 85 registers spill ~100 bytes.
 // ROOMY: one block, for launches of at most one block per SM, where a second
 // has nothing to run; the registers go into four couples per iteration, whose
