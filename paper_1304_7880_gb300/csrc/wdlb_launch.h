@@ -47,7 +47,7 @@ struct BatchGroup {
     int nitems;
 };
 
-constexpr int kMaxBatchGroups = 16;
+constexpr int kMaxBatchGroups = 24;   // 18 tiled variants, and generic ones with and without walls and split
 
 // Device tables of a multi-lattice step.  bufs[p]: one KBufs per slot (of the
 // launcher's storage type), input buffer = the slot's buffer for parity p.
