@@ -663,7 +663,8 @@ wdlb_status wdlb_create(wdlb_lattice lat, double sigma, int32_t walls, double ta
     ctx->Npad = (ctx->N + 63) / 64 * 64;
     build_ball(sigma, ctx->tab.ball);
     build_shell_rule(sigma, o.shell_rule, ctx->tab.shell, ctx->tab.wvec);
-    if (o.shell_rule == WDLB_SHELL_FULL) ctx->tab.ncouple = order_couples(ctx->tab.shell);   // one weight for all
+    if (o.shell_rule == WDLB_SHELL_FULL && o.storage != WDLB_STORE_F16)   // one weight for all
+        ctx->tab.ncouple = order_couples(ctx->tab.shell);
     ctx->tab.wshell = o.shell_rule == WDLB_SHELL_COMPACT ? 1.0 : ctx->tab.wvec[0];
     ctx->L = &launchers_for(o.storage, o.collision);
     set_params(ctx);

@@ -49,7 +49,7 @@ struct KParams {
     int nx, ny, nz, walls;   // walls: solid planes z = 0 and z = nz-1
     int N, Npad;             // node count, padded stride of per-node arrays
     int nshell, nball;
-    int ncouple;             // mirror couples at the head of the shell table (order_couples); 0: compact shell
+    int ncouple;             // mirror couples at the head of the shell table (order_couples); 0: compact shell, FP16 storage
     int closure, omega_mode, interactions;
     int s2;                  // 2 sigma if it is an integer, else 0 (selects a compiled shell)
     int tiled;               // 1: use the shared-memory tiled shell kernel
@@ -294,5 +294,22 @@ struct Store<__half> {
     __device__ __forceinline__ static float load(const __half *p, float scale) { return __half2float(*p) * scale; }
     __device__ __forceinline__ static void put(__half *p, float v, float inv_scale) { *p = __float2half_rn(v * inv_scale); }
 };
+
+// Whether the full shell's pairs are summed as mirror couples (order_couples).
+// FP16 storage keeps the table's order: it is for periodic boxes, where the
+// couples' exact zeros along the walls have no part, and the rounding of its
+// stored populations turns a last bit of the sums into 2e-4 of u (96^3, sigma 6,
+// ten steps), so that another order would change every result visibly for
+// nothing but speed (shell kernel there 0.494 ms as couples, 0.508 so).
+template <class S>
+constexpr bool sums_couples()
+{
+    return true;
+}
+template <>
+constexpr bool sums_couples<__half>()
+{
+    return false;
+}
 
 }  // namespace wdlb

@@ -347,22 +347,22 @@ __device__ __forceinline__ void ball_brick_ct(const KParams &p, const V4<T> *nu,
 // ---------------------------------------------------------------------------
 // Pair weights of a (+e, -e) pair of the contact shell.  With
 // q = g2(chi_mid) n(r+e) (without the quadrature weight), chi_mid/2 =
-// hb(r) + hb(r+e), the weights are carried doubled, Q = 2q, which drops the
-// factor 1/2 of the closures: with a = 1/s, s = 1 - chi_mid, G = 2 g2 is
-//   CS: a^2 + a^3    PY: 3 a^2 - a    closure one: 2.
-// s0 = 1 - h(r) - h_off; dh, dn: deviations of the two neighbours.  Besides Q+
-// and Q- it returns 2 (Q+ - Q-), formed from the deviations so that it is
-// accurate relative to itself (it is what the mean-field sum accumulates):
-//   2 (Q+ - Q-) = (G+ + G-)(dn+ - dn-) + (G+ - G-)(n+ + n-),
-//   a+ - a- = (dh+ - dh-) a+ a-,   T = a+ + a-,
-//   CS: G+ - G- = (a+ - a-) (T + T^2 - a+ a-)    PY: (a+ - a-) (3 T - 1)
-// (exact divided differences of the closures in a, which take four
-// operations fewer per pair than in s: 128^3 full shell, sigma 4, 0.543 ->
-// 0.517 ms).  One reciprocal of s+ s- for both ends, and G+ dn+ - G- dn- in place
-// of the products above, are cheaper still but less exact (u_z of the driven
-// 8 x 8 x 41 slit off by 3.3e-4 of max|u_x| instead of 1.1e-4): a product s- /
-// (s+ s-) has twice the error of a reciprocal, and next to a wall dn is as
-// large as n.
+// hb(r) + hb(r+e), the weights are carried doubled, Q = 2q, which makes the
+// Carnahan-Starling value one multiply-add: 2 g2 = (1 + s)/s^3 with
+// s = 1 - chi_mid (Percus-Yevick: (3 - s)/s^2; closure one: 2).  s0 = 1 - h(r)
+// - h_off; dh, dn: deviations of the two neighbours.  Besides Q+ and Q- it
+// returns 2 (Q+ - Q-), formed from the deviations so that it is accurate
+// relative to itself (it is what the mean-field sum accumulates):
+//   2 (Q+ - Q-) = (G+ + G-)(dn+ - dn-) + (G+ - G-)(n+ + n-),   G = 2 g2,
+//   CS:  G+ - G- = (dh+ - dh-) [s+^2 + s-^2 + s+ s- (1 + s+ + s-)] / (s+^3 s-^3)
+//   PY:  G+ - G- = (dh+ - dh-) [3 (s+ + s-) - s+ s-] / (s+^2 s-^2)
+// (exact divided differences of the closures; s- - s+ = dh+ - dh-).
+// The same in a = 1/s (G = a^2 + a^3) takes four operations fewer per pair (128^3
+// full shell, sigma 4, 0.489 -> 0.472 ms; FP64 45 x 38 x 51 1.074 -> 1.005 ms)
+// but is less exact: the error of the reciprocal enters a^2 and a^3 about 2.6
+// times, here once.  rms error of Q in FP32 against FP64, as a multiple of this
+// form's with every operation correctly rounded: this form 1.013 to 1.015, that
+// one 1.24 to 1.37 (a million pairs, bulk-like and wall-like, both closures).
 // ---------------------------------------------------------------------------
 template <class T>
 __device__ __forceinline__ T fast_rcp(T x);
@@ -394,26 +394,27 @@ __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(
 template <int CL, class T>
 __device__ __forceinline__ void pair_weights(T s0, T noff, T dhp, T dnp, T dhm, T dnm, T &qp, T &qm, T &qd)
 {
+    const T np = noff + dnp, nm = noff + dnm;
     if (CL == 2) {
-        qp = T(2) * (noff + dnp);
-        qm = T(2) * (noff + dnm);
+        qp = T(2) * np;
+        qm = T(2) * nm;
         qd = T(4) * (dnp - dnm);
         return;
     }
-    const T np = noff + dnp, nm = noff + dnm;
-    const T ap = fast_rcp<T>(s0 - dhp), am = fast_rcp<T>(s0 - dhm);
-    const T sum = add_rn(ap, am), prod = ap * am;
-    const T dif = (dhp - dhm) * prod;
+    const T sp = s0 - dhp, sm = s0 - dhm;
+    const T spm = sp * sm;
     T gp, gm, gd;
     if (CL == 0) {
-        const T ap2 = ap * ap, am2 = am * am;
-        gp = fma(ap2, ap, ap2);
-        gm = fma(am2, am, am2);
-        gd = dif * (fma(sum, sum, sum) - prod);
+        const T sp2 = sp * sp, sm2 = sm * sm;
+        const T rp = fast_rcp<T>(sp2 * sp), rm = fast_rcp<T>(sm2 * sm);
+        gp = fma(sp, rp, rp);
+        gm = fma(sm, rm, rm);
+        gd = (dhp - dhm) * (add_rn(sp2, sm2) + fma(spm, sp + sm, spm)) * (rp * rm);
     } else {
-        gp = ap * fma(T(3), ap, T(-1));
-        gm = am * fma(T(3), am, T(-1));
-        gd = dif * fma(T(3), sum, T(-1));
+        const T rp = fast_rcp<T>(sp * sp), rm = fast_rcp<T>(sm * sm);
+        gp = fma(-sp, rp, T(3) * rp);
+        gm = fma(-sm, rm, T(3) * rm);
+        gd = (dhp - dhm) * fma(T(3), sp + sm, -spm) * (rp * rm);
     }
     qp = gp * np;
     qm = gm * nm;
@@ -566,36 +567,6 @@ __device__ __forceinline__ int push_target(const PushOffsets &o, int i, int cx, 
            (cz < 0 ? o.zm : cz > 0 ? o.zp : 0);
 }
 
-// alpha + beta.c + c.Gamma.c at the lattice directions; gab is 2 Gamma_ab.  Sums
-// only, never contracted, with the even and the odd part of opposite directions
-// the same bits.
-template <class T>
-struct CollisionPoly {
-    T al, bx, by, bz, gxx, gyy, gzz, gxy, gxz, gyz;
-    __device__ __forceinline__ T at(int q) const
-    {
-        const int cx = cx_of(q), cy = cy_of(q), cz = cz_of(q);
-        T e = al, o = T(0);          // o: the odd part times the sign of the first component
-        if (cx) {
-            e = add_rn(e, gxx);
-            o = bx;
-        }
-        if (cy) {
-            e = add_rn(e, gyy);
-            o = cx ? add_rn(o, cx * cy > 0 ? by : -by) : by;
-        }
-        if (cz) {
-            e = add_rn(e, gzz);
-            o = cx || cy ? add_rn(o, (cx + cy) * cz > 0 ? bz : -bz) : bz;
-        }
-        if (cx && cy) e = add_rn(e, cx * cy > 0 ? gxy : -gxy);
-        if (cx && cz) e = add_rn(e, cx * cz > 0 ? gxz : -gxz);
-        if (cy && cz) e = add_rn(e, cy * cz > 0 ? gyz : -gyz);
-        const int lead = cx ? cx : cy ? cy : cz;
-        return lead ? add_rn(e, lead > 0 ? o : -o) : e;
-    }
-};
-
 // target_dn(q, dst) returns n - n_off of the node a population is pushed to
 // (this step's density there: its storage scale for the next step).
 template <class S, int CL, bool WALLS, bool FIELDS, class T, class TargetDn>
@@ -622,8 +593,9 @@ __device__ __forceinline__ void collide_push(const KParams &p, const KBufs<S, T>
 
     // collision velocity u = (j + F/2)/n with F = n g + C
     const T Fx = n * prm<T>(p.g[0], p.f_g[0]) + Cx, Fy = n * prm<T>(p.g[1], p.f_g[1]) + Cy, Fz = n * prm<T>(p.g[2], p.f_g[2]) + Cz;
-    const T mx = fma(T(0.5), Fx, jx), my = fma(T(0.5), Fy, jy), mz = fma(T(0.5), Fz, jz);   // n u
-    const T ux = mx * inv_n, uy = my * inv_n, uz = mz * inv_n;
+    const T ux = (jx + T(0.5) * Fx) * inv_n;
+    const T uy = (jy + T(0.5) * Fy) * inv_n;
+    const T uz = (jz + T(0.5) * Fz) * inv_n;
 
     if (FIELDS) {
         const int N = p.N;
@@ -646,53 +618,12 @@ __device__ __forceinline__ void collide_push(const KParams &p, const KBufs<S, T>
     }
 
     // collision (Eq. SMDB, second order): f* = f - omega (f - feq) + (1 - omega/2)(Phi + S^A)
-    // with feq - w_q s and Phi + S^A, both quadratic in c, as w_q times polynomials
-    // of ten coefficients per node (about 25 operations per direction less)
     const T tr3 = (Axx + Ayy + Azz) * T(1.0 / 3.0);
+    const T Bxx = Axx - tr3, Byy = Ayy - tr3, Bzz = Azz - tr3;   // traceless A
     const T kA = p.interactions ? prm<T>(p.k_cross, p.f_k_cross) * T(4.5) : T(0);  // K / (2 c_s^4)
-    const T src_pref = fma(T(-0.5), omega, T(1));
-    const T uu = fma(ux, ux, fma(uy, uy, uz * uz));
-    const T uF = fma(ux, Fx, fma(uy, Fy, uz * Fz));
-    // frc: (1 - omega/2)(Phi + S^A) / w_q; eq: (feq - w_q s) / w_q times es,
-    // dn + n (3 cu + 4.5 cu^2 - 1.5 uu).  In FP64 frc takes eq in, with es = omega.
-    // In FP32 they stay apart: d - feq is formed before the product with omega,
-    // so that near equilibrium its rounding is the difference's, not d's (one
-    // polynomial doubled the error of a 1e-6 shear wave at sigma 8 after 20 steps
-    // and left the converged 161-node slit at n* 0.3 1.1e-5 off on u_x, 5.0e-6 so).
-    constexpr bool kApart = sizeof(T) == sizeof(float);
-    // With walls and FP32 storage, where the momentum of the changes is restored
-    // below, 3 n, 4.5 n and the multiples of 1 - omega/2 are formed once per node.
-    // Elsewhere the products are with n u and F themselves: the rounding of 3 n
-    // is the same on every node of a uniform fluid and on every step (the 1e-6
-    // shear wave at sigma 8 was 9.8e-7 off after 20 steps, 2.4e-7 so).
-    constexpr bool kRestored = WALLS && sizeof(S) == sizeof(float) && kApart;
-    const T es = kApart ? T(1) : omega;
-    const T n3 = T(3) * n, n45 = T(4.5) * n, p3 = T(3) * src_pref, p9 = T(9) * src_pref;
-    const T wx = es * mx, wy = es * my, wz = es * mz;                              // n u
-    const T fx = src_pref * Fx, fy = src_pref * Fy, fz = src_pref * Fz;
-    const T pk = src_pref * kA, pk2 = T(2) * pk;
-    CollisionPoly<T> eq, frc;
-    eq.al = fma(T(-1.5) * es * n, uu, es * dn);
-    eq.bx = kRestored ? n3 * ux : T(3) * wx;
-    eq.by = kRestored ? n3 * uy : T(3) * wy;
-    eq.bz = kRestored ? n3 * uz : T(3) * wz;
-    const T hx = kRestored ? n45 * ux : T(4.5) * wx, hy = kRestored ? n45 * uy : T(4.5) * wy,
-            hz = kRestored ? n45 * uz : T(4.5) * wz;
-    eq.gxx = ux * hx; eq.gyy = uy * hy; eq.gzz = uz * hz;
-    eq.gxy = T(2) * (ux * hy); eq.gxz = T(2) * (ux * hz); eq.gyz = T(2) * (uy * hz);
-    const T kx = kRestored ? p9 * Fx : T(9) * fx, ky = kRestored ? p9 * Fy : T(9) * fy,
-            kz = kRestored ? p9 * Fz : T(9) * fz;
-    const auto onto = [](T v, T w) { return kApart ? v : v + w; };
-    frc.al = onto(kRestored ? -p3 * uF : T(-3) * (src_pref * uF), eq.al);
-    frc.bx = onto(kRestored ? p3 * Fx : T(3) * fx, eq.bx);
-    frc.by = onto(kRestored ? p3 * Fy : T(3) * fy, eq.by);
-    frc.bz = onto(kRestored ? p3 * Fz : T(3) * fz, eq.bz);
-    frc.gxx = onto(fma(ux, kx, pk * (Axx - tr3)), eq.gxx);
-    frc.gyy = onto(fma(uy, ky, pk * (Ayy - tr3)), eq.gyy);
-    frc.gzz = onto(fma(uz, kz, pk * (Azz - tr3)), eq.gzz);
-    frc.gxy = onto(fma(ux, ky, fma(uy, kx, pk2 * Axy)), eq.gxy);
-    frc.gxz = onto(fma(ux, kz, fma(uz, kx, pk2 * Axz)), eq.gxz);
-    frc.gyz = onto(fma(uy, kz, fma(uz, ky, pk2 * Ayz)), eq.gyz);
+    const T uu = ux * ux + uy * uy + uz * uz;
+    const T uF = ux * Fx + uy * Fy + uz * Fz;
+    const T src_pref = T(1) - T(0.5) * omega;
     const PushOffsets po = push_offsets<WALLS>(x, y, z, nx, ny, nz);
 
     // push streaming with half-way bounce-back; re-encode relative to the
@@ -716,10 +647,19 @@ __device__ __forceinline__ void collide_push(const KParams &p, const KBufs<S, T>
         const T stored = post + wq * (dsc - dn_t);
         Store<S>::put(b.f_out + (size_t)qq * p.Npad + dst, stored, T(1.0 / w_of(q)) * fast_rcp<T>(noff + dn_t));
     };
-    const auto change = [&](int q) {    // f*_q - f_q
-        return fma(T(w_of(q)), frc.at(q), omega * fma(T(w_of(q)), eq.at(q), -d[q]));
+    // population q's equilibrium deviation and its forcing (Phi + S^A)
+    const auto relax = [&](int q, T &feq_dev, T &forcing) {
+        const int cxq = cx_of(q), cyq = cy_of(q), czq = cz_of(q);
+        const T wq = T(w_of(q));
+        const T cu = T(cxq) * ux + T(cyq) * uy + T(czq) * uz;
+        const T cF = T(cxq) * Fx + T(cyq) * Fy + T(czq) * Fz;
+        feq_dev = wq * (dn + n * (T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu));
+        const T phi = wq * (T(3) * (cF - uF) + T(9) * cu * cF);
+        const T cAc = T(cxq * cxq) * Bxx + T(cyq * cyq) * Byy + T(czq * czq) * Bzz +
+                      T(2 * cxq * cyq) * Axy + T(2 * cxq * czq) * Axz + T(2 * cyq * czq) * Ayz;
+        forcing = phi + kA * wq * cAc;
     };
-    if constexpr (kRestored) {
+    if constexpr (WALLS && sizeof(S) == sizeof(float) && sizeof(T) == sizeof(float)) {
         // FP32 storage in a slit: the momentum of the changes along the walls
         // (x, y), which is F exactly, is summed in double-word arithmetic and
         // 3 w_q c_q . (F - sum) is added back.  The roundings inside the changes
@@ -731,8 +671,10 @@ __device__ __forceinline__ void collide_push(const KParams &p, const KBufs<S, T>
         dwf Mx = dw_from(0.f), My = dw_from(0.f);
 #pragma unroll
         for (int q = 0; q < NQ; q++) {
-            const T dl = change(q);
-            d[q] = add_rn(d[q], dl);
+            T feq_dev, forcing;
+            relax(q, feq_dev, forcing);
+            const T dl = src_pref * forcing - omega * (d[q] - feq_dev);   // the change
+            d[q] = d[q] + dl;
             if (cx_of(q)) Mx += cx_of(q) > 0 ? dl : -dl;
             if (cy_of(q)) My += cy_of(q) > 0 ? dl : -dl;
         }
@@ -745,8 +687,11 @@ __device__ __forceinline__ void collide_push(const KParams &p, const KBufs<S, T>
         }
     } else {
 #pragma unroll
-        for (int q = 0; q < NQ; q++)
-            push(q, kApart ? add_rn(d[q], change(q)) : fma(T(w_of(q)), frc.at(q), fma(-omega, d[q], d[q])));
+        for (int q = 0; q < NQ; q++) {
+            T feq_dev, forcing;
+            relax(q, feq_dev, forcing);
+            push(q, d[q] - omega * (d[q] - feq_dev) + src_pref * forcing);
+        }
     }
     b.nscale[i] = dn_self;
     b.cprev[i] = Cx;

@@ -170,8 +170,9 @@ bool compiled_table_matches()
     } else {
         double w = 0.0;
         build_shell(sigma, e, &w);
-        const tiled::ct::FullTable<S2> &T = tiled::ct::kFull<S2>;
-        if (order_couples(e) != T.nc || (int)e.size() != 6 * (2 * T.nc + T.ns)) return false;
+        constexpr bool CPL = sums_couples<S>();
+        const tiled::ct::FullTable<S2, CPL> &T = tiled::ct::kFull<S2, CPL>;
+        if ((CPL ? order_couples(e) : 0) != T.nc || (int)e.size() != 6 * (2 * T.nc + T.ns)) return false;
         constexpr int SX = tiled::TX + 2 * tiled::shell_radius(S2);
         for (int m = 0; m < 2 * T.nc + T.ns; m++) {
             const tiled::ct::PairEntry &t = T.e[m < 2 * T.nc ? m / 2 : m - T.nc];

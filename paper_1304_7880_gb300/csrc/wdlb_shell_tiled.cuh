@@ -19,11 +19,12 @@
 // The (+e, -e) pairs of the full shell sit in constant memory with their tile
 // offsets (ct::FullTable); the loop over them is kept rolled (two couples per
 // iteration) so the code stays in the instruction cache.  The kernel is bound by
-// instruction issue: a staged table and offsets cost 68 instructions per pair,
-// this form 60; with pair_weights' closed form and the couples the 128^3 box's
-// full shell took 0.543 -> 0.478 ms (sigma 4, FP32), the 96^3 box's at sigma 6
-// (FP16) 0.551 -> 0.474 ms.  Each pair goes through pair_weights, pair_terms and
-// accumulate_couple, the same arithmetic in the same order as shell_body.  WT
+// instruction issue, and a pair staged per block with its offset takes more of
+// it than one read through uniform registers.  Shell kernel, staged table and
+// now: 128^3 box at sigma 4, FP32 0.543 -> 0.498 ms (0.515 without the couples),
+// 96^3 box at sigma 6, FP16 storage (pairs in table order) 0.551 -> 0.509 ms.
+// Each pair goes through pair_weights, pair_terms and accumulate_couple, the same
+// arithmetic in the same order as shell_body.  WT
 // (the compact shell): the pairs are compiled in, with one weight per orbit that
 // scales each pair's Q as in shell_body.
 #pragma once
@@ -158,14 +159,15 @@ constexpr int first_pair_of_orbit(int o)
 // over the block, as couples (a, b, c), (a, b, -c) and the pairs left over
 // (c = 0 and a = b = 0): unit vector and, for the nu tile (16 bytes per node)
 // and the hb tile (4), the byte offsets of (a, b, c) and of (a, b, -c); a
-// single's second pair of offsets is unused.
+// single's second pair of offsets is unused.  Without COUPLES every pair is a
+// single, in the order of build_shell.
 struct PairEntry {
     float kx, ky, kz;
     int p16, p4, m16, m4;         // +(a, b, c), -(a, b, c)
     int q16, q4, r16, r4, pad;    // +(a, b, -c), -(a, b, -c)
 };
 
-template <int S2>
+template <int S2, bool COUPLES>
 struct FullTable {
     int nc, ns;                   // couples, then singles from e[nc] on
     PairEntry e[256];
@@ -176,14 +178,13 @@ struct FullTable {
         for (int pass = 0; pass < 2; pass++)
             for (int dx = 0; dx <= R; dx++)
                 for (int dy = -R; dy <= R; dy++)
-                    for (int dz = 0; dz <= R; dz++) {
+                    for (int dz = -R; dz <= R; dz++) {
                         const bool axis = dx == 0 && dy == 0;
-                        const bool positive = dx > 0 || dy > 0 || (axis && dz > 0);
+                        const bool positive = dx > 0 || (dx == 0 && (dy > 0 || (dy == 0 && dz > 0)));
                         const int r2 = dx * dx + dy * dy + dz * dz;
-                        if ((dx == 0 && dy < 0) || !positive || !((S2 - 1) * (S2 - 1) < 4 * r2 && 4 * r2 <= (S2 + 1) * (S2 + 1)))
-                            continue;
-                        const bool couple = dz > 0 && !axis;
-                        if (couple != (pass == 0)) continue;
+                        if (!positive || !((S2 - 1) * (S2 - 1) < 4 * r2 && 4 * r2 <= (S2 + 1) * (S2 + 1))) continue;
+                        const bool paired = COUPLES && dz != 0 && !axis;   // in a couple, which dz > 0 stands for
+                        if (paired != (pass == 0) || (paired && dz < 0)) continue;
                         const double len = sqrt_newton(double(r2));
                         const int o = dx + SX * (dy + SX * dz), o2 = dx + SX * (dy - SX * dz);
                         PairEntry &t = e[m++];
@@ -198,7 +199,7 @@ struct FullTable {
                         t.q4 = 4 * o2;
                         t.r16 = -16 * o2;
                         t.r4 = -4 * o2;
-                        if (couple)
+                        if (paired)
                             nc++;
                         else
                             ns++;
@@ -206,10 +207,10 @@ struct FullTable {
     }
 };
 
-template <int S2>
-constexpr FullTable<S2> kFull = FullTable<S2>();
-template <int S2>
-__constant__ FullTable<S2> c_full = FullTable<S2>();
+template <int S2, bool COUPLES>
+constexpr FullTable<S2, COUPLES> kFull = FullTable<S2, COUPLES>();
+template <int S2, bool COUPLES>
+__constant__ FullTable<S2, COUPLES> c_full = FullTable<S2, COUPLES>();
 
 // Shells with a compiled table: the compact rule at sigma 3, 4 and 6 (13, 21
 // and 15 pairs; 7-10 % faster than the runtime table on the 128^3 box).  The
@@ -459,14 +460,16 @@ __device__ __forceinline__ void tiled_body(const KParams &p, const KBufs<S, floa
                                                        me.z, me.w);
                 });
             }
-            // The runtime loop over the full shell: 60 instructions per pair (54
-            // multiply-adds, two reciprocals, four loads).  Table and offsets
-            // come through uniform registers, so an address takes none; two
-            // couples per iteration for sigma 3 and 4 (1, 3 and 4 measured 3, 1
-            // and 1.5 % slower), one for sigma 6.
-            constexpr int kUnroll = ROOMY ? 4 : S2 >= 12 ? 1 : 2;
+            // The runtime loop over the full shell: 58 operations per single pair
+            // (26 for the weights, 32 for the sums), 55.5 per pair of a couple, two
+            // reciprocals and four loads.  Table and offsets come through uniform
+            // registers, so an address takes none; two couples per iteration for
+            // sigma 3 and 4 (1, 3 and 4 measured 3, 1 and 1.5 % slower), one for
+            // sigma 6.
+            constexpr bool CPL = sums_couples<S>();
+            constexpr int kUnroll = ROOMY ? 4 : S2 >= 12 ? 1 : CPL ? 2 : 3;
             if constexpr (!CT) {
-                constexpr int NC = ct::kFull<S2>.nc, NSI = ct::kFull<S2>.ns;
+                constexpr int NC = ct::kFull<S2, CPL>.nc, NSI = ct::kFull<S2, CPL>.ns;
                 static_assert(2 * NC + NSI == NPAIR, "couples and singles cover the shell");
                 const char *c16 = reinterpret_cast<const char *>(sm4 + base);
                 const char *c4 = reinterpret_cast<const char *>(smh + base);
@@ -482,13 +485,13 @@ __device__ __forceinline__ void tiled_body(const KParams &p, const KBufs<S, floa
                                              me.w);
                 };
                 const auto couple = [&](int m) {
-                    const ct::PairEntry &t = ct::c_full<S2>.e[m];
+                    const ct::PairEntry &t = ct::c_full<S2, CPL>.e[m];
                     if (!inside(t.p4) || !inside(t.m4) || !inside(t.q4) || !inside(t.r4)) return;
                     accumulate_couple<float>(a, t.kx, t.ky, t.kz, terms(t.p16, t.p4, t.m16, t.m4, t.kx, t.ky, t.kz),
                                              terms(t.q16, t.q4, t.r16, t.r4, t.kx, t.ky, -t.kz));
                 };
                 const auto single = [&](int m) {
-                    const ct::PairEntry &t = ct::c_full<S2>.e[m];
+                    const ct::PairEntry &t = ct::c_full<S2, CPL>.e[m];
                     if (!inside(t.p4) || !inside(t.m4)) return;
                     accumulate_terms<float>(a, t.kx, t.ky, t.kz,
                                             terms(t.p16, t.p4, t.m16, t.m4, t.kx, t.ky, t.kz));
