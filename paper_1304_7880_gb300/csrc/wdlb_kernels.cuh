@@ -936,7 +936,7 @@ __device__ __forceinline__ void shell_body(const KParams &p, const KBufs<S, type
 // ---------------------------------------------------------------------------
 constexpr int kSplit = 4;   // (eight: 96^3 at sigma 8 1 607 -> 2 149 us, FP64 45 x 38 x 51 1 055 -> 1 369)
 
-template <class S, int CL, bool WALLS, bool WT, class A = typename Store<S>::T>
+template <class S, int CL, bool WALLS, bool FIELDS, bool WT, class A = typename Store<S>::T>
 __device__ __forceinline__ void shell_split_body(const KParams &p, const KBufs<S, typename Store<S>::T> &b, int node0)
 {
     typedef typename Store<S>::T T;
@@ -1008,18 +1008,32 @@ __device__ __forceinline__ void shell_split_body(const KParams &p, const KBufs<S
     if (p.interactions)
         shell_forces<T>(p, a, noff + me.x, me.y, me.z, me.w, Cx, Cy, Cz, Axx, Ayy, Azz, Axy, Axz, Ayz, tsum);
     const auto target_dn = [&](int, int dst) { return in_bounds(dst, p.N, b.status) ? b.nu[dst].x : T(0); };
-    if constexpr (is_dw<A>::value)
+    if constexpr (is_dw<A>::value && !FIELDS)
         collide_push_dw<S, CL, WALLS>(p, b, i, x, y, z, hr, Cx, Cy, Cz, Axx, Ayy, Azz, Axy, Axz, Ayz, tsum, me.x,
                                       target_dn);
     else
-        collide_push<S, CL, WALLS, false>(p, b, i, x, y, z, hr, Cx, Cy, Cz, Axx, Ayy, Azz, Axy, Axz, Ayz, tsum, me.x,
-                                          target_dn);
+        collide_push<S, CL, WALLS, FIELDS>(p, b, i, x, y, z, hr, Cx, Cy, Cz, Axx, Ayy, Azz, Axy, Axz, Ayz, tsum, me.x,
+                                           target_dn);
 }
 
+// Fields of the current state (no step), one node per thread or, where the step
+// splits a node's pairs, in the same four partial sums: the collision velocity
+// u = (j + F/2)/n is a small difference next to a wall (j_z against F_z/2), so
+// F has to be the step's own, bit for bit.
 template <class S, int CL, bool WALLS, bool FIELDS, bool WT>
 __global__ void __launch_bounds__(256) k_shell_collide(KParams p, KBufs<S, typename Store<S>::T> b)
 {
     shell_body<S, CL, WALLS, FIELDS, WT>(p, b, blockIdx.x);
+}
+
+// the split forms: kSplitBlocks blocks of 32 nodes per 256 nodes
+constexpr int kSplitBlocks = 8;
+
+template <class S, int CL, bool WALLS, bool WT>
+__global__ void __launch_bounds__(32 * kSplit) k_shell_fields_split(KParams p, KBufs<S, typename Store<S>::T> b)
+{
+    if (32 * (int)blockIdx.x >= p.N) return;
+    shell_split_body<S, CL, WALLS, true, WT>(p, b, 32 * (int)blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------

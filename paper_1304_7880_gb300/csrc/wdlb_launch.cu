@@ -58,13 +58,22 @@ KBufs<S, T> typed(const DevBufs &d, int cur)
     return b;
 }
 
+template <int CL, bool WALLS, bool WT>
+void launch_fields_rule(const KParams &p, const KBufs<S, T> &b, cudaStream_t st)
+{
+    if (!p.tiled && p.split)
+        k_shell_fields_split<S, CL, WALLS, WT><<<blocks_for(p.N) * kSplitBlocks, 32 * kSplit, 0, st>>>(p, b);
+    else
+        k_shell_collide<S, CL, WALLS, true, WT><<<blocks_for(p.N), kThreads, 0, st>>>(p, b);
+}
+
 template <int CL, bool WALLS>
 void launch_fields_shell(const KParams &p, const KBufs<S, T> &b, cudaStream_t st)
 {
     if (p.shell_rule)
-        k_shell_collide<S, CL, WALLS, true, true><<<blocks_for(p.N), kThreads, 0, st>>>(p, b);
+        launch_fields_rule<CL, WALLS, true>(p, b, st);
     else
-        k_shell_collide<S, CL, WALLS, true, false><<<blocks_for(p.N), kThreads, 0, st>>>(p, b);
+        launch_fields_rule<CL, WALLS, false>(p, b, st);
 }
 
 #if WDLB_STORAGE != 0

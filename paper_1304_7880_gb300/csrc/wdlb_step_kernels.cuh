@@ -60,8 +60,6 @@ __global__ void __launch_bounds__(256) k_step_shell(const KParams *P, const KBuf
 }
 
 // the split form: kSplitBlocks blocks of 32 nodes per work item of 256 nodes
-constexpr int kSplitBlocks = 8;
-
 template <class S, int CL, bool WALLS, bool WT, class A = typename Store<S>::T>
 __global__ void __launch_bounds__(32 * kSplit)
     k_step_shell_split(const KParams *P, const KBufs<S, typename Store<S>::T> *B, const BatchItem *it)
@@ -71,7 +69,7 @@ __global__ void __launch_bounds__(32 * kSplit)
     const KParams p = P[w.slot];
     if (node0 >= p.N) return;
     const KBufs<S, typename Store<S>::T> b = B[w.slot];
-    shell_split_body<S, CL, WALLS, WT, A>(p, b, node0);
+    shell_split_body<S, CL, WALLS, false, WT, A>(p, b, node0);
 }
 
 template <class S, int S2, int V, bool WALLS, bool WT, class A = float, bool ROOMY = false>
