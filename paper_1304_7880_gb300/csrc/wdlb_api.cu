@@ -263,17 +263,21 @@ wdlb_status check_status_word(wdlb_ctx *ctx)
 
 // Whether the generic shell kernel splits a node's pairs over four warps (one
 // fourth of the sum each, then one warp for the collision).  Splitting pays
-// wherever the sums outweigh the collision, which three of the four warps sit
-// out: always on the full shells (31 pairs at sigma 2 and more), and on any
-// shell while the lattice leaves SMs without a block of 256 nodes.  Shell
-// kernel, unsplit against split, us: sigma 8 full FP32 256.6 / 36.9 on 4 096
-// nodes, 2 321 / 1 500 on 96^3; sigma 3 full (PY) 325 / 291 on 96^3; sigma 4
-// full FP64 585 / 92 on 4 096 nodes, 1 697 / 1 531 on 48^3.  Sigma 8 compact
-// (21 pairs): 20.6 / 11.9 on 16 384 nodes, 20.5 / 20.6 on 36 864, 178 / 228 on
-// 96^3; in FP64 at sigma 4 156 / 109 and 156 / 166 on the first two.
-int split_shell(int npair, long long N)
+// where the sums outweigh the collision, which three of the four warps sit out:
+// with 31 pairs and more, the full shells from sigma 2 on.  In FP64, where both
+// forms share one FP64 pipe, it pays on small lattices from 19 pairs on, the
+// larger compact shells.  Elsewhere it is faster only while a lattice has the GPU
+// to itself: many such pores of a batch fill it together, and the rule looks at
+// one lattice (a pore keeps its bits alone and in a batch).  Shell kernel, unsplit
+// against split, us.  Pays: sigma 7.5 full FP32 2 098 / 1 248 on 96^3; sigma 2
+// full FP32 (31 pairs) 216 / 218 on 96^3, 76 / 67 on 64^3, 317 / 269 on 64 pores
+// of 16 384 nodes; sigma 4 compact FP64 (21 pairs) 147 / 104 on 16 384 nodes, 3 787
+// / 3 684 on 64 of them, 156 / 166 on 36 864.  Does not: sigma 8 compact FP32 (21)
+// 18.6 / 12.4 on 16 384 nodes, but 232 / 292 on 64 of them; sigma 1.5 full FP32
+// (13) 14 / 10 and 169 / 215; sigma 3 compact FP64 (13) 2 771 / 2 933 on 64.
+int split_shell(int storage, int npair, long long N)
 {
-    return npair >= 31 || N <= 24576 ? 1 : 0;
+    return npair >= 31 || (storage == WDLB_STORE_F64 && npair >= 19 && N <= 24576) ? 1 : 0;
 }
 
 void set_params(wdlb_ctx *ctx)
@@ -311,7 +315,7 @@ void set_params(wdlb_ctx *ctx)
     p.tiled = 0;
     p.shell_r = 0;
     for (int c : ctx->tab.shell) p.shell_r = std::max(p.shell_r, std::abs(c));
-    p.split = split_shell(p.nshell / 2, ctx->N);
+    p.split = split_shell(ctx->opt.storage, p.nshell / 2, ctx->N);
     p.ball_r = 0;
     for (size_t m = 0; m < ctx->tab.ball.size(); m++) p.ball_r = std::max(p.ball_r, std::abs(ctx->tab.ball[m]));
     const size_t tsize = ctx->opt.storage == WDLB_STORE_F64 ? sizeof(double) : sizeof(float);
@@ -663,7 +667,9 @@ wdlb_status wdlb_create(wdlb_lattice lat, double sigma, int32_t walls, double ta
     ctx->Npad = (ctx->N + 63) / 64 * 64;
     build_ball(sigma, ctx->tab.ball);
     build_shell_rule(sigma, o.shell_rule, ctx->tab.shell, ctx->tab.wvec);
-    if (o.shell_rule == WDLB_SHELL_FULL && o.storage != WDLB_STORE_F16)   // one weight for all
+    // couples need one weight for all pairs; the unsplit generic kernel keeps the table's order
+    if (o.shell_rule == WDLB_SHELL_FULL && o.storage != WDLB_STORE_F16 &&
+        split_shell(o.storage, (int)ctx->tab.shell.size() / 6, ctx->N))
         ctx->tab.ncouple = order_couples(ctx->tab.shell);
     ctx->tab.wshell = o.shell_rule == WDLB_SHELL_COMPACT ? 1.0 : ctx->tab.wvec[0];
     ctx->L = &launchers_for(o.storage, o.collision);

@@ -822,7 +822,7 @@ __device__ __forceinline__ void collide_push_dw(const KParams &p, const KBufs<S,
 // walls.  nu, hb in deviation form (see above).  WT: per-vector quadrature
 // weights (the compact shell) in shell_k[m].w scale the pair's Q; without
 // WT the uniform weight is applied once, in shell_forces.
-template <int CL, bool WALLS, class T, bool WT = false>
+template <int CL, bool WALLS, class T, bool WT = false, bool COUPLES = false>
 __device__ __forceinline__ void shell_sums_generic(const KParams &p, const V4<T> *nu, const T *hb,
                                                    const int4 *shell_e, const V4<T> *shell_k, int x, int y, int z,
                                                    T hr, T vx, T vy, T vz, ShellAcc<T> &a, int *status)
@@ -861,12 +861,15 @@ __device__ __forceinline__ void shell_sums_generic(const KParams &p, const V4<T>
         return pair_terms<T>(k.x, k.y, k.z, qp, qm, qd, nb[0].y, nb[0].z, nb[0].w, nb[1].y, nb[1].z, nb[1].w, vx, vy,
                              vz);
     };
-    const int nc = WT ? 0 : 4 * p.ncouple;
-    for (int m = 0; m < nc; m += 4) {               // mirror couples, as in the tiled kernel
-        const int4 e = shell_e[m];
-        const V4<T> k = shell_k[m];
-        accumulate_couple<T>(a, k.x, k.y, k.z, terms(e, k),
-                             terms(make_int4(e.x, e.y, -e.z, 0), V4<T>{k.x, k.y, -k.z, k.w}));
+    int nc = 0;
+    if constexpr (COUPLES) {                        // mirror couples, as in the tiled kernel
+        nc = 4 * p.ncouple;
+        for (int m = 0; m < nc; m += 4) {
+            const int4 e = shell_e[m];
+            const V4<T> k = shell_k[m];
+            accumulate_couple<T>(a, k.x, k.y, k.z, terms(e, k),
+                                 terms(make_int4(e.x, e.y, -e.z, 0), V4<T>{k.x, k.y, -k.z, k.w}));
+        }
     }
     for (int m = nc; m + 1 < p.nshell; m += 2) {
         const V4<T> k = shell_k[m];
@@ -902,8 +905,9 @@ __device__ __forceinline__ void shell_body(const KParams &p, const KBufs<S, type
     T tsum = T(0);
     if (p.interactions) {
         ShellAcc<T> a = {};
-        shell_sums_generic<CL, WALLS, T, WT>(p, b.nu, b.hb, b.shell_e, b.shell_k, x, y, z, hr, vx, vy, vz, a,
-                                             b.status);
+        // couples: the fields pass of a lattice that steps in the tiled kernel
+        shell_sums_generic<CL, WALLS, T, WT, FIELDS && !WT>(p, b.nu, b.hb, b.shell_e, b.shell_k, x, y, z, hr, vx, vy,
+                                                            vz, a, b.status);
         shell_forces<T>(p, a, n, vx, vy, vz, Cx, Cy, Cz, Axx, Ayy, Azz, Axy, Axz, Ayz, tsum);
     }
     const auto target_dn = [&](int, int dst) { return in_bounds(dst, p.N, b.status) ? b.nu[dst].x : T(0); };
