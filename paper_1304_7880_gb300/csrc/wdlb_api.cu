@@ -319,7 +319,7 @@ void set_params(wdlb_ctx *ctx)
     p.ball_r = 0;
     for (size_t m = 0; m < ctx->tab.ball.size(); m++) p.ball_r = std::max(p.ball_r, std::abs(ctx->tab.ball[m]));
     const size_t tsize = ctx->opt.storage == WDLB_STORE_F64 ? sizeof(double) : sizeof(float);
-    p.ball_tiled = ball_tile_smem(p.ball_r, p.nball, tsize) <= kBallTileMaxSmem ? 1 : 0;
+    p.ball_tiled = ball_tile_smem(p.s2, p.ball_r, p.nball, tsize) <= kBallTileMaxSmem ? 1 : 0;
     // n_off / ref_ng are set at init (they may depend on the initial state)
 }
 
@@ -390,10 +390,12 @@ cudaError_t upload_step_tables(wdlb_ctx *ctx)
     blocks();
     LL.n_node_items = nb;
     if (p.ball_tiled) {
-        LL.ball_items = dit + items.size();
+        const bool ct = ball_compiled(p.s2);
+        (ct ? LL.ball_items : LL.ball_offset_items) = dit + items.size();
         bricks(kBallTile);
-        LL.n_ball_items = tx * ty * tz;
-        LL.ball_smem = ball_tile_smem(p.ball_r, p.nball, ctx->opt.storage == WDLB_STORE_F64 ? 8 : 4);
+        (ct ? LL.n_ball_items : LL.n_ball_offset_items) = tx * ty * tz;
+        (ct ? LL.ball_smem : LL.ball_offset_smem) =
+            ball_tile_smem(p.s2, p.ball_r, p.nball, ctx->opt.storage == WDLB_STORE_F64 ? 8 : 4);
     } else {
         LL.ball_node_items = dit + items.size();
         blocks();
@@ -1313,8 +1315,8 @@ wdlb_status batch_build(wdlb_batch *b)
     std::vector<KParams> params(P);
     std::vector<StatSlot> stat(P, StatSlot{nullptr, nullptr, nullptr, nullptr});
     std::vector<char> bufs0(b->L->kbufs_bytes * P, 0), bufs1(b->L->kbufs_bytes * P, 0);
-    std::vector<BatchItem> node_items, ball_items, ball_node_items;
-    size_t ball_smem = 0;
+    std::vector<BatchItem> node_items, ball_items, ball_offset_items, ball_node_items;
+    size_t ball_smem = 0, ball_offset_smem = 0;
     struct Key {
         int s2, walls, tiled, closure, tile, rule, split;
         bool operator<(const Key &o) const
@@ -1336,11 +1338,14 @@ wdlb_status batch_build(wdlb_batch *b)
         if (c->kp.ball_tiled) {
             const int bt = kBallTile;
             const int tx = (c->lat.nx + bt - 1) / bt, ty = (c->lat.ny + bt - 1) / bt, tz = (c->lat.nz + bt - 1) / bt;
+            const bool ct = ball_compiled(c->kp.s2);
+            auto &list = ct ? ball_items : ball_offset_items;
             for (int z = 0; z < tz; z++)
                 for (int y = 0; y < ty; y++)
-                    for (int x = 0; x < tx; x++) ball_items.push_back(BatchItem{s, x, y, z});
+                    for (int x = 0; x < tx; x++) list.push_back(BatchItem{s, x, y, z});
             const size_t tsize = c->opt.storage == WDLB_STORE_F64 ? sizeof(double) : sizeof(float);
-            ball_smem = std::max(ball_smem, ball_tile_smem(c->kp.ball_r, c->kp.nball, tsize));
+            size_t &smem = ct ? ball_smem : ball_offset_smem;
+            smem = std::max(smem, ball_tile_smem(c->kp.s2, c->kp.ball_r, c->kp.nball, tsize));
         } else {
             for (int k = 0; k < (N + 255) / 256; k++) ball_node_items.push_back(BatchItem{s, k, 0, 0});
         }
@@ -1358,7 +1363,7 @@ wdlb_status batch_build(wdlb_batch *b)
         }
     }
     if ((int)groups.size() > kMaxBatchGroups) return bfail(b, WDLB_ERR_ARG, "too many kernel variants in one batch");
-    size_t total = node_items.size() + ball_items.size() + ball_node_items.size();
+    size_t total = node_items.size() + ball_items.size() + ball_offset_items.size() + ball_node_items.size();
     for (auto &g : groups) total += g.second.size();
     if (total > b->items_cap) {
         if (b->d_items) cudaFree(b->d_items);
@@ -1380,6 +1385,10 @@ wdlb_status batch_build(wdlb_batch *b)
     L.n_ball_items = (int)ball_items.size();
     L.ball_smem = ball_smem;
     all.insert(all.end(), ball_items.begin(), ball_items.end());
+    L.ball_offset_items = b->d_items + all.size();
+    L.n_ball_offset_items = (int)ball_offset_items.size();
+    L.ball_offset_smem = ball_offset_smem;
+    all.insert(all.end(), ball_offset_items.begin(), ball_offset_items.end());
     L.ball_node_items = b->d_items + all.size();
     L.n_ball_node_items = (int)ball_node_items.size();
     all.insert(all.end(), ball_node_items.begin(), ball_node_items.end());
@@ -1404,6 +1413,7 @@ wdlb_status batch_build(wdlb_batch *b)
     std::vector<int> counts(3 * size_t(std::max(P, 1)), 0);
     for (const BatchItem &it : node_items) counts[3 * it.slot + 0]++;
     for (const BatchItem &it : ball_items) counts[3 * it.slot + 1]++;
+    for (const BatchItem &it : ball_offset_items) counts[3 * it.slot + 1]++;
     for (auto &g : groups)
         for (const BatchItem &it : g.second) counts[3 * it.slot + 2]++;
     if (P > 0 && b->flow)

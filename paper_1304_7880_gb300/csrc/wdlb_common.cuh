@@ -10,8 +10,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <algorithm>
-
 namespace wdlb {
 
 constexpr int NQ = 19;
@@ -117,7 +115,7 @@ __device__ __forceinline__ float prm<float>(double, float f) { return f; }
 constexpr int kMaxShellR = 8;    // floor(sigma + 1/2) for sigma <= 8
 
 // Tiled ball sum: an 8 x 8 x 8 brick of nodes per block with a halo of
-// ball_r, the brick's n - n_off and the ball's offsets (or the brick's
+// ball_r, the brick's n - n_off and the ball's offsets (compiled balls: the brick's
 // row indices, side^2) in shared memory.
 constexpr int kBallTile = 8;
 constexpr int kBallThreads = 256;
@@ -134,10 +132,15 @@ inline __host__ __device__ constexpr int ball_pitch(int side, size_t tsize)
     return side <= 24 && size_t(side) * side * (24 * tsize + sizeof(int)) <= kBallTileMaxSmem ? 24 : side;
 }
 
-inline size_t ball_tile_smem(int ball_r, int nball, size_t tsize)
+// Whether the ball of 2 sigma = s2 is compiled into the tiled kernel (the pitch
+// and the row indices are that form's; any other sigma holds offsets at run time).
+inline __host__ __device__ bool ball_compiled(int s2) { return s2 == 6 || s2 == 8 || s2 == 12 || s2 == 16; }
+
+inline size_t ball_tile_smem(int s2, int ball_r, int nball, size_t tsize)
 {
     const size_t side = size_t(kBallTile + 2 * ball_r);
-    return side * side * ball_pitch((int)side, tsize) * tsize + std::max(size_t(nball), side * side) * sizeof(int);
+    return ball_compiled(s2) ? side * side * (ball_pitch((int)side, tsize) * tsize + sizeof(int))
+                             : side * side * side * tsize + size_t(nball) * sizeof(int);
 }
 
 // Device buffers of one lattice.  S: storage type of populations; T: compute type.

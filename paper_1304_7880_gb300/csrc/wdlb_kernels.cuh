@@ -192,7 +192,8 @@ __device__ __forceinline__ void ball_body(const KParams &p, const V4<T> *nu, T *
     hb[i] = dh;
 }
 
-// Tiled form of ball_body: one 8 x 8 x 8 brick of nodes per block, with n - n_off of the brick
+// Tiled form of ball_body: one 8 x 8 x 8 brick of nodes per block of 256
+// threads (two nodes per thread, z and z + 4), with n - n_off of the brick
 // and its halo of ball_r, and the ball's offsets within it, in shared memory.
 // Beyond a wall the staged value is -n_off (n = 0).  The brick arrives by
 // cp.async (all of a thread's loads in flight at once).  The ball points are
@@ -228,8 +229,9 @@ __device__ __forceinline__ void ball_tiled_body(const KParams &p, const V4<T> *n
     }
     cp_async_wait_all();
     __syncthreads();
-    const int tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7;
-    for (int tz = threadIdx.x >> 6; tz < kBallTile; tz += blockDim.x >> 6) {
+    const int tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7, tzb = threadIdx.x >> 6;
+    for (int half = 0; half < 2; half++) {
+        const int tz = tzb + 4 * half;
         const int x = x0 + tx, y = y0 + ty, z = z0 + tz;
         if (x >= p.nx || y >= p.ny || z >= p.nz) continue;
         const int i = x + p.nx * (y + p.ny * z);

@@ -332,6 +332,11 @@ cudaError_t do_batch_step(const BatchLaunch &L, int parity, int part, int group,
             k_step_ball_tiled<S><<<L.n_ball_items, kBallThreads, L.ball_smem, st>>>(L.params, B, L.ball_items);
             *launches += 1;
         }
+        if (L.n_ball_offset_items > 0) {
+            k_step_ball_offsets<S><<<L.n_ball_offset_items, kThreads, L.ball_offset_smem, st>>>(L.params, B,
+                                                                                               L.ball_offset_items);
+            *launches += 1;
+        }
         if (L.n_ball_node_items > 0) {
             k_step_ball<S><<<L.n_ball_node_items, kThreads, 0, st>>>(L.params, B, L.ball_node_items);
             *launches += 1;
@@ -378,7 +383,7 @@ cudaError_t do_batch_step(const BatchLaunch &L, int parity, int part, int group,
 bool do_flow_ok(const BatchLaunch &L)
 {
 #if WDLB_STORAGE != 0
-    if (L.n_ball_node_items != 0 || L.ngroups != 1 || L.n_ball_items == 0) return false;
+    if (L.n_ball_node_items != 0 || L.n_ball_offset_items != 0 || L.ngroups != 1 || L.n_ball_items == 0) return false;
     const BatchGroup &G = L.groups[0];
     return G.tiled && G.s2 == 8 && G.tile == 2 && G.closure == 0 && G.nitems > 0;
 #else

@@ -56,9 +56,12 @@ struct BatchLaunch {
     const void *bufs[2];
     const BatchItem *node_items;      // blocks of 256 nodes of every slot (moments)
     int n_node_items;
-    const BatchItem *ball_items;      // 8^3 bricks of the slots with a tiled ball sum
+    const BatchItem *ball_items;      // 8^3 bricks of the slots with a compiled ball (ball_compiled)
     int n_ball_items;
-    size_t ball_smem;                 // largest tiled ball shared memory among them
+    size_t ball_smem;                 // largest shared memory among them
+    const BatchItem *ball_offset_items;   // bricks of the slots with a tiled ball sum of another sigma
+    int n_ball_offset_items;
+    size_t ball_offset_smem;
     const BatchItem *ball_node_items; // blocks of 256 nodes of the other slots
     int n_ball_node_items;
     BatchGroup groups[kMaxBatchGroups];

@@ -32,9 +32,10 @@ __global__ void __launch_bounds__(256) k_step_ball(const KParams *P, const KBufs
     ball_body<typename Store<S>::T>(p, b.nu, b.hb, b.ball, b.status, w.bx);
 }
 
+// bricks of the lattices whose ball is compiled in
 template <class S>
-__global__ void __launch_bounds__(kBallThreads) k_step_ball_tiled(const KParams *P, const KBufs<S, typename Store<S>::T> *B,
-                                                         const BatchItem *it)
+__global__ void __launch_bounds__(kBallThreads)
+    k_step_ball_tiled(const KParams *P, const KBufs<S, typename Store<S>::T> *B, const BatchItem *it)
 {
     const BatchItem w = it[blockIdx.x];
     const KParams p = P[w.slot];
@@ -44,9 +45,22 @@ __global__ void __launch_bounds__(kBallThreads) k_step_ball_tiled(const KParams 
     case 6: ball_brick_ct<T, 6, kBallThreads>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
     case 8: ball_brick_ct<T, 8, kBallThreads>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
     case 12: ball_brick_ct<T, 12, kBallThreads>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
-    case 16: ball_brick_ct<T, 16, kBallThreads>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
-    default: ball_tiled_body<T>(p, b.nu, b.hb, b.ball, b.status, w.bx, w.by, w.bz); break;
+    default: ball_brick_ct<T, 16, kBallThreads>(p, b.nu, b.hb, b.status, w.bx, w.by, w.bz); break;
     }
+}
+
+// Bricks of the other lattices.  A kernel of its own: compiled together with the
+// bricks above, its loop kept fewer loads in flight (smeared density of 96^3,
+// FP32, sigma 2 18.6 us, sigma 5 35.0; alone 16.8 and 32.7; 64^3 in FP64, sigma 1
+// 12.3 and 10.3).
+template <class S>
+__global__ void __launch_bounds__(256)
+    k_step_ball_offsets(const KParams *P, const KBufs<S, typename Store<S>::T> *B, const BatchItem *it)
+{
+    const BatchItem w = it[blockIdx.x];
+    const KParams p = P[w.slot];
+    const KBufs<S, typename Store<S>::T> b = B[w.slot];
+    ball_tiled_body<typename Store<S>::T>(p, b.nu, b.hb, b.ball, b.status, w.bx, w.by, w.bz);
 }
 
 template <class S, int CL, bool WALLS, bool WT, class A = typename Store<S>::T>
