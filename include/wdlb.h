@@ -144,8 +144,9 @@ typedef struct {
                                  wdlb_batch_step call in which each pore's phases
                                  follow one another without device-wide barriers
                                  (used where every pore runs the tiled sigma-4 kernel
-                                 on 8 x 8 x 4 bricks, else the default).  Both give
-                                 bitwise the same results                            */
+                                 on 8 x 8 x 4 bricks, which such a batch's pores take
+                                 unless tile forces a shape; else the default).  Both
+                                 give bitwise the same results                       */
     int32_t collision;        /* arithmetic of the collision and push (step 3 of
                                  Sec. 5, Eq. SMDB) with FP32 storage:
                                  WDLB_COLLISION_FP32 (default) FP32; with walls
@@ -315,7 +316,8 @@ wdlb_status wdlb_profile_step(wdlb_ctx *ctx, int64_t nsteps, double ms[3]);
  * scratch lattice of that key (nz as given, a square cross-section of about
  * 2^20 / nz nodes so that the kernel fills the GPU as a batch does; uniform
  * density; six steps after two warm-up steps) when autotune = 1, else from a
- * built-in table.  Every shape computes the same arithmetic per node; alone
+ * built-in table, whose shape also stays where no other is faster by more than
+ * the probe's noise.  Every shape computes the same arithmetic per node; alone
  * and batched lattices of one key share the table entry, so they run the
  * same kernel.  Thread-safe; the table lives until wdlb_autotune_reset. */
 

@@ -296,25 +296,25 @@ constexpr bool tma_staging()
 
 // Blocks per SM the launch bounds ask for: for 256 threads, three where three
 // blocks' shared memory fits (227 KB per SM; the compiler then keeps to 85
-// registers per thread), else two where two fit, else one.  Three blocks
-// measured 7-12 % faster than two for sigma 3 (8^3 bricks) and sigma 4 (8 x 8 x 4 bricks), and 5 % faster for the double-word
-// collision at sigma 4, whose 85 registers spill ~100 bytes.
+// registers per thread), else two where two fit, else one; one for 512
+// threads.  Three blocks measured 7-12 % faster than two for sigma 3 (8^3
+// bricks) and sigma 4 (8 x 8 x 4 bricks), and 5 % faster for the double-word
+// collision at sigma 4, whose 85 registers spill ~100 bytes.  Two blocks of 512
+// threads (64 registers, spills) only draw level with the 256-thread shapes at
+// sigma 3 and 4 (128^3 full shell 0.507 ms against 0.497, compact 0.201 against
+// 0.199), which left the choice between them to the probe's noise.
 // ROOMY: one block, for launches of at most one block per SM, where a second
 // has nothing to run; the registers go into four couples per iteration, whose
-// loads and reciprocals overlap (8 x 8 x 41 slit, sigma 4: 50 steps 1.16 -> 1.09
-// ms; 27 x 27 x 46, sigma 3, 96 bricks: 100 steps 2.55 -> 2.38 ms; on 128^3
-// 0.474 -> 0.481 ms).  The sums are the same bits.
-// 512 threads: two blocks where two fit (32 warps at 64 registers; compact shell
-// at sigma 4 on 128^3 0.255 -> 0.188 ms, the 256-thread shapes 0.196; full shell
-// 0.561 -> 0.471), one with the double-word collision, which would spill.
-template <int S2, int V, bool ROOMY = false, bool DW = false>
+// loads and reciprocals overlap (shell kernel of the 8 x 8 x 41 slit, sigma 4, 20.5
+// -> 19.4 us; 27 x 27 x 46, sigma 3, 96 bricks, 21.1 -> 19.7 us).  The sums are
+// the same bits.
+template <int S2, int V, bool ROOMY = false>
 constexpr int blocks_per_sm()
 {
-    return ROOMY || (threads_of(V) != 256 && DW)               ? 1
-           : threads_of(V) != 256                              ? (2 * smem_bytes<S2, V>() <= size_t(227) * 1024 ? 2 : 1)
+    return ROOMY || threads_of(V) != 256                   ? 1
            : 3 * smem_bytes<S2, V>() <= size_t(227) * 1024 ? 3
            : 2 * smem_bytes<S2, V>() <= size_t(227) * 1024 ? 2
-                                                                : 1;
+                                                           : 1;
 }
 
 template <class S, int S2, int V, int CL, bool WALLS, bool FIELDS, bool WT = false, class A = float,

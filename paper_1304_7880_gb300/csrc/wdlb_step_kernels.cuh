@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(32 * kSplit)
 }
 
 template <class S, int S2, int V, bool WALLS, bool WT, class A = float, bool ROOMY = false>
-__global__ void __launch_bounds__(tiled::threads_of(V), (tiled::blocks_per_sm<S2, V, ROOMY, is_dw<A>::value>()))
+__global__ void __launch_bounds__(tiled::threads_of(V), (tiled::blocks_per_sm<S2, V, ROOMY>()))
     k_step_shell_tiled(const KParams *P, const KBufs<S, float> *B, const BatchItem *it)
 {
     const BatchItem w = it[blockIdx.x];
