@@ -170,7 +170,7 @@ bool compiled_table_matches()
     if constexpr (WT) {
         std::vector<double> wts;
         if (!build_shell_compact(sigma, e, wts)) return false;
-        constexpr tiled::ct::PairTable<S2, WT> T{};
+        constexpr tiled::ct::PairTable<S2> T{};
         if ((int)e.size() != 6 * T.n) return false;
         for (int m = 0; m < T.n; m++) {
             if (e[6 * m] != T.ex[m] || e[6 * m + 1] != T.ey[m] || e[6 * m + 2] != T.ez[m]) return false;

@@ -58,14 +58,17 @@ constexpr int shell_count(int S2)
 }
 
 // ---------------------------------------------------------------------------
-// Compile-time shell tables.  For the shells below, the (+e, -e) pairs are
-// generated at compile time in the order of the library's table (dx from 0 to
-// R, then dy and dz from -R to R, +e lexicographically positive), so the pair
-// loop unrolls with constant unit vectors and constant tile offsets, and the
-// products with a zero component of khat drop out.  The compact rule's orbits
-// (sorted |components|) at sigma 3, 4 and 6 are the ones the library's rule
-// selects; wdlb_launch.cu checks the library's table against these before it
-// uses them.  The per-orbit weights stay runtime values.
+// Compile-time shell tables.  The compact shell's (+e, -e) pairs (13, 21 and 15
+// at sigma 3, 4 and 6) are generated at compile time in the order of the library's
+// table (dx from 0 to R, then dy and dz from -R to R, +e lexicographically
+// positive), so the pair loop unrolls with constant unit vectors and constant tile
+// offsets, and the products with a zero component of khat drop out (7-10 % faster
+// than a run-time table on the 128^3 box).  The compact rule's orbits (sorted
+// |components|) at sigma 3, 4 and 6 are the ones the library's rule selects;
+// wdlb_launch.cu checks the library's table against these before it uses them.
+// The per-orbit weights stay runtime values.  The full shells keep a rolled loop
+// (FullTable): unrolled, their 49 to 225 pairs ran 4 % (sigma 3) and 21 % (sigma 4)
+// slower, the code no longer fitting the instruction cache.
 // ---------------------------------------------------------------------------
 namespace ct {
 
@@ -76,7 +79,7 @@ constexpr double sqrt_newton(double x)
     return r;
 }
 
-constexpr int kMaxPairs = 128;
+constexpr int kMaxPairs = 32;   // of a compact shell
 
 struct Orbits {
     int n;
@@ -109,7 +112,7 @@ constexpr int orbit_of(int S2, int x, int y, int z)
     return -1;
 }
 
-template <int S2, bool COMPACT>
+template <int S2>
 struct PairTable {
     int n;
     int ex[kMaxPairs], ey[kMaxPairs], ez[kMaxPairs], orb[kMaxPairs];
@@ -122,7 +125,7 @@ struct PairTable {
                     const bool positive = dx > 0 || (dx == 0 && (dy > 0 || (dy == 0 && dz > 0)));
                     const int r4 = 4 * (dx * dx + dy * dy + dz * dz);
                     if (!positive || !((S2 - 1) * (S2 - 1) < r4 && r4 <= (S2 + 1) * (S2 + 1))) continue;
-                    const int o = COMPACT ? orbit_of(S2, dx, dy, dz) : 0;
+                    const int o = orbit_of(S2, dx, dy, dz);
                     if (o < 0 || n >= kMaxPairs) continue;
                     ex[n] = dx;
                     ey[n] = dy;
@@ -134,10 +137,10 @@ struct PairTable {
 };
 
 // largest |component| of the table's vectors
-template <int S2, bool COMPACT>
+template <int S2>
 constexpr int max_component()
 {
-    constexpr PairTable<S2, COMPACT> T{};
+    constexpr PairTable<S2> T{};
     int mx = 0;
     for (int m = 0; m < T.n; m++) {
         const int c[3] = {T.ex[m], T.ey[m], T.ez[m]};
@@ -149,7 +152,7 @@ constexpr int max_component()
 template <int S2>
 constexpr int first_pair_of_orbit(int o)
 {
-    constexpr PairTable<S2, true> T{};
+    constexpr PairTable<S2> T{};
     for (int m = 0; m < T.n; m++)
         if (T.orb[m] == o) return m;
     return 0;
@@ -167,10 +170,24 @@ struct PairEntry {
     int q16, q4, r16, r4, pad;    // +(a, b, -c), -(a, b, -c)
 };
 
+// number of couples of a full shell (pairs of (a, b, c > 0), (a, b) != (0, 0))
+constexpr int couple_count(int S2)
+{
+    const int R = shell_radius(S2);
+    int m = 0;
+    for (int dx = 0; dx <= R; dx++)
+        for (int dy = dx ? -R : 1; dy <= R; dy++)
+            for (int dz = 1; dz <= R; dz++) {
+                const int r4 = 4 * (dx * dx + dy * dy + dz * dz);
+                if ((S2 - 1) * (S2 - 1) < r4 && r4 <= (S2 + 1) * (S2 + 1)) m++;
+            }
+    return m;
+}
+
 template <int S2, bool COUPLES>
 struct FullTable {
     int nc, ns;                   // couples, then singles from e[nc] on
-    PairEntry e[256];
+    PairEntry e[shell_count(S2) / 2 - (COUPLES ? couple_count(S2) : 0)];
     constexpr FullTable() : nc(0), ns(0), e{}
     {
         const int R = (S2 + 1) / 2, SX = 8 + 2 * R;
@@ -211,17 +228,6 @@ template <int S2, bool COUPLES>
 constexpr FullTable<S2, COUPLES> kFull = FullTable<S2, COUPLES>();
 template <int S2, bool COUPLES>
 __constant__ FullTable<S2, COUPLES> c_full = FullTable<S2, COUPLES>();
-
-// Shells with a compiled table: the compact rule at sigma 3, 4 and 6 (13, 21
-// and 15 pairs; 7-10 % faster than the runtime table on the 128^3 box).  The
-// full shells keep the runtime loop: unrolled, their 49 to 225 pairs ran 4 %
-// (sigma 3) and 21 % (sigma 4) slower, the code no longer fitting the
-// instruction cache.
-template <int S2, bool COMPACT>
-constexpr bool compiled()
-{
-    return COMPACT && compact_orbits(S2).n > 0;
-}
 
 template <int B, int E, class F>
 __device__ __forceinline__ void static_for(F &&f)
@@ -328,23 +334,23 @@ __device__ __forceinline__ void tiled_body(const KParams &p, const KBufs<S, floa
     constexpr int NPAIR = shell_count(S2) / 2;
     constexpr int NT = threads_of(V);
     constexpr int ZSTEP = NT / (TX * TY);     // z rows covered by one pass of the block
-    // shared memory: nu tile (16 B per node), hb tile (4 B per node), pair
-    // table, pair weights, mbarrier; the two tiles 128-byte aligned for TMA
+    // shared memory: nu tile (16 B per node), hb tile (4 B per node), mbarrier;
+    // the two tiles 128-byte aligned for TMA
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float4 *sm4 = reinterpret_cast<float4 *>(smem_raw);
     float *smh = reinterpret_cast<float *>(smem_raw + sizeof(float4) * NS);
     uint64_t *bar = reinterpret_cast<uint64_t *>(
         smem_raw + smem_bytes<S2, V>() - sizeof(uint64_t));
     static_assert(((sizeof(float4) + sizeof(float)) * NS) % 8 == 0, "mbarrier alignment");
-    constexpr bool CT = ct::compiled<S2, WT>();
+    static_assert(!WT || ct::compact_orbits(S2).n > 0, "per-vector weights need a compiled table");
 
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const int x0 = bx * TX, y0 = by * TY, z0 = bz * TZ;
 
-    // compiled table with the compact rule: the weight of each orbit, taken
+    // compact shell: the weight of each orbit, taken
     // from the first pair of the orbit in the library's table
     float wo[3] = {1.f, 1.f, 1.f};
-    if constexpr (CT && WT) {
+    if constexpr (WT) {
         ct::static_for<0, ct::compact_orbits(S2).n>([&](auto O) {
             constexpr int m = ct::first_pair_of_orbit<S2>(decltype(O)::value);
             wo[decltype(O)::value] = b.shell_k[2 * m].w;
@@ -433,13 +439,13 @@ __device__ __forceinline__ void tiled_body(const KParams &p, const KBufs<S, floa
         if (p.interactions) {
             ShellAcc<float> a = {};
             const float s0 = 1.f - hr - hoff;
-            if constexpr (CT) {
-                constexpr ct::PairTable<S2, WT> T{};
+            if constexpr (WT) {
+                constexpr ct::PairTable<S2> T{};
                 // The offsets are constants: every component of a table vector
                 // is at most R, the tile's halo, so base +- off stays inside the
                 // tile for every thread.  Proved here at compile time, which
                 // keeps the pair loop the same code in the checked build.
-                static_assert(ct::max_component<S2, WT>() <= R, "shell vector beyond the tile halo");
+                static_assert(ct::max_component<S2>() <= R, "shell vector beyond the tile halo");
                 ct::static_for<0, T.n>([&](auto M) {
                     constexpr int m = decltype(M)::value;
                     constexpr int EX = T.ex[m], EY = T.ey[m], EZ = T.ez[m];
@@ -450,12 +456,10 @@ __device__ __forceinline__ void tiled_body(const KParams &p, const KBufs<S, floa
                     const float hm = smh[base - off];
                     float qp, qm, qd;
                     pair_weights<CL, float>(s0, noff, hp, np.x, hm, nm.x, qp, qm, qd);
-                    if constexpr (WT) {
-                        const float r = wo[T.orb[m]];
-                        qp *= r;
-                        qm *= r;
-                        qd *= r;
-                    }
+                    const float r = wo[T.orb[m]];
+                    qp *= r;
+                    qm *= r;
+                    qd *= r;
                     ct::accumulate_pair_ct<EX, EY, EZ>(a, qp, qm, qd, np.y, np.z, np.w, nm.y, nm.z, nm.w, me.y,
                                                        me.z, me.w);
                 });
@@ -468,7 +472,7 @@ __device__ __forceinline__ void tiled_body(const KParams &p, const KBufs<S, floa
             // sigma 6.
             constexpr bool CPL = sums_couples<S>();
             constexpr int kUnroll = ROOMY ? 4 : S2 >= 12 ? 1 : CPL ? 2 : 3;
-            if constexpr (!CT) {
+            if constexpr (!WT) {
                 constexpr int NC = ct::kFull<S2, CPL>.nc, NSI = ct::kFull<S2, CPL>.ns;
                 static_assert(2 * NC + NSI == NPAIR, "couples and singles cover the shell");
                 const char *c16 = reinterpret_cast<const char *>(sm4 + base);
