@@ -338,6 +338,13 @@ wdlb_status wdlb_tile_info(const wdlb_ctx *ctx, int32_t *tiled, int32_t *tile);
  * 0 if every brick copies it node by node.  No counterpart in the paper. */
 wdlb_status wdlb_staging_info(const wdlb_ctx *ctx, int32_t *tma);
 
+/* Which form of its shell kernel a context runs when it is stepped alone:
+ * *split 1 if the per-node kernel splits a node's pairs over four warps,
+ * *roomy 1 if the tiled full-shell kernel takes the form for launches of at
+ * most one block per SM (the same bits as the other form).  No counterpart in
+ * the paper. */
+wdlb_status wdlb_shell_info(const wdlb_ctx *ctx, int32_t *split, int32_t *roomy);
+
 /* Forget every autotuned entry (later contexts probe again). */
 void wdlb_autotune_reset(void);
 
@@ -398,6 +405,9 @@ wdlb_ctx *wdlb_batch_context(wdlb_batch *b, int32_t slot);
 int32_t wdlb_batch_active(const wdlb_batch *b);
 uint64_t wdlb_batch_free_bytes(const wdlb_batch *b);
 int64_t wdlb_batch_launch_count(const wdlb_batch *b);
+/* Shell launches per step of the batch as it was last stepped, and how many of
+ * them run the split and the roomy form (wdlb_shell_info); any may be NULL. */
+wdlb_status wdlb_batch_shell_info(const wdlb_batch *b, int32_t *launches, int32_t *split, int32_t *roomy);
 const char *wdlb_batch_last_error(const wdlb_batch *b);
 void wdlb_batch_destroy(wdlb_batch *b);
 

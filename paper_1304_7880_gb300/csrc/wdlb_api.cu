@@ -1186,6 +1186,14 @@ wdlb_status wdlb_staging_info(const wdlb_ctx *ctx, int32_t *tma)
     return WDLB_OK;
 }
 
+wdlb_status wdlb_shell_info(const wdlb_ctx *ctx, int32_t *split, int32_t *roomy)
+{
+    if (!ctx || !split || !roomy) return WDLB_ERR_ARG;
+    *split = ctx->launch.groups[0].split;
+    *roomy = ctx->launch.groups[0].roomy;
+    return WDLB_OK;
+}
+
 void wdlb_autotune_reset(void)
 {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
@@ -1804,6 +1812,20 @@ uint64_t wdlb_batch_free_bytes(const wdlb_batch *b)
 }
 
 int64_t wdlb_batch_launch_count(const wdlb_batch *b) { return b ? b->launches : 0; }
+
+wdlb_status wdlb_batch_shell_info(const wdlb_batch *b, int32_t *launches, int32_t *split, int32_t *roomy)
+{
+    if (!b) return WDLB_ERR_ARG;
+    int32_t ns = 0, nr = 0;
+    for (int g = 0; g < b->launch.ngroups; g++) {
+        ns += b->launch.groups[g].split;
+        nr += b->launch.groups[g].roomy;
+    }
+    if (launches) *launches = b->launch.ngroups;
+    if (split) *split = ns;
+    if (roomy) *roomy = nr;
+    return WDLB_OK;
+}
 
 const char *wdlb_batch_last_error(const wdlb_batch *b) { return b ? b->err.c_str() : g_create_error.c_str(); }
 

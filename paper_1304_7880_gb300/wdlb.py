@@ -114,6 +114,8 @@ def load_library(path: str = LIB_PATH):
         "wdlb_fields_static": (I32, [wdlb_lattice, D, I32, I32, P, P, P, P, P, P]),
         "wdlb_launch_count": (I64, [P]),
         "wdlb_staging_info": (I32, [P, P]),
+        "wdlb_shell_info": (I32, [P, P, P]),
+        "wdlb_batch_shell_info": (I32, [P, P, P, P]),
         "wdlb_last_error": (ctypes.c_char_p, [P]),
         "wdlb_batch_create": (I32, [P, ctypes.c_uint64, I32, P]),
         "wdlb_batch_pore_bytes": (I32, [P, P, P]),
@@ -349,6 +351,13 @@ def wdlb_staging_info(ctx: Context) -> bool:
     return bool(tma.value)
 
 
+def wdlb_shell_info(ctx: Context):
+    """(split, roomy): the form of its shell kernel a context runs alone."""
+    split, roomy = ctypes.c_int32(), ctypes.c_int32()
+    _check(load_library().wdlb_shell_info(ctx.handle, ctypes.byref(split), ctypes.byref(roomy)), ctx)
+    return bool(split.value), bool(roomy.value)
+
+
 def wdlb_autotune_reset():
     load_library().wdlb_autotune_reset()
 
@@ -489,7 +498,7 @@ def _bcheck(status, batch=None):
 
 def wdlb_batch_create(max_pores, pool_bytes, closure="CS", omega_mode="const", storage="f32", interactions=True,
                       k_cross=2.0, device=None, shell_rule="full", autotune=True, staging="auto",
-                      persistent=False, wait_limit=0, collision="fp32"):
+                      persistent=False, wait_limit=0, collision="fp32", tile=-1):
     import torch
 
     lib = load_library()
@@ -506,6 +515,7 @@ def wdlb_batch_create(max_pores, pool_bytes, closure="CS", omega_mode="const", s
     opt.staging = STAGINGS[staging]
     opt.persistent = 1 if persistent else 0
     opt.wait_limit = int(wait_limit)
+    opt.tile = int(tile)
     dev = torch.device(device) if device is not None else torch.device("cuda", torch.cuda.current_device())
     pool = torch.empty(int(pool_bytes) + 256, dtype=torch.uint8, device=dev)
     stream = torch.cuda.Stream(device=dev)
@@ -587,6 +597,13 @@ def wdlb_batch_free_bytes(batch) -> int:
 
 def wdlb_batch_launch_count(batch) -> int:
     return int(load_library().wdlb_batch_launch_count(batch.handle))
+
+
+def wdlb_batch_shell_info(batch):
+    """(launches, split, roomy): shell launches per step, and those of either form."""
+    v = [ctypes.c_int32() for _ in range(3)]
+    _check(load_library().wdlb_batch_shell_info(batch.handle, *(ctypes.byref(x) for x in v)))
+    return tuple(x.value for x in v)
 
 
 def wdlb_batch_destroy(batch):
