@@ -25,8 +25,10 @@
  *   dd  all of it in double.
  * Nodes within `band` layers of a wall take the variant `band_mode`, the rest
  * `inner_mode`.  `qd` picks the form of Q+ - Q- in the mean-field sum: sym (the
- * kernel's, odd under swapping the pair's ends bit for bit) or asym (the
- * earlier form, which rounds differently at the two ends).
+ * kernel's, odd under swapping the pair's ends bit for bit), asym (the
+ * earlier form, which rounds differently at the two ends), both with the pairs
+ * summed one by one in table order, or couple: sym summed in the kernel's order,
+ * (a, b, c) together with (a, b, -c) and then the pairs left over.
  *
  *   column <nz> <n*> <sigma> <tau> <g_x> <steps> <band> <band_mode> <inner_mode> <qd>
  *
@@ -48,12 +50,12 @@
 static int C[Q][3];
 static double W[Q];
 static int OPP[Q];
-static int NZ, NP, NB, BZ[64], PE[128][3];
+static int NZ, NE, NB, BZ[64], PE[128][3], PC[128];   /* NE entries; PC: 1 a couple, 0 a pair */
 static double SIG, TAU, GX, PK[128][3], WSH, NOFF, HOFF, CHIN, CHALF, BETA, HPRED, SIG2;
 static STORE *f[2][Q], *nudn, *nuv[3], *hb, *cprev[3], *tprev;
 static double *nscale;
 static int cur = 0;
-static int QD_ASYM = 0;
+static int QD_ASYM = 0, COUPLES = 0;
 static double XF_INNER, XF_DRIVE;
 
 /* D3Q19 in the library's order: rest, faces, edges (Sec. 5). */
@@ -77,19 +79,22 @@ static void tables(void)
 {
     int R = (int)floor(SIG + 0.5);
     double lo = (SIG - 0.5) * (SIG - 0.5), hi = (SIG + 0.5) * (SIG + 0.5), second = 0;
-    NP = 0;
-    for (int dx = 0; dx <= R; dx++)
-        for (int dy = -R; dy <= R; dy++)
-            for (int dz = -R; dz <= R; dz++) {
-                int pos = dx > 0 || (dx == 0 && (dy > 0 || (dy == 0 && dz > 0)));
-                double r2 = dx * dx + dy * dy + dz * dz;
-                if (!pos || !(r2 > lo && r2 <= hi)) continue;
-                double L = sqrt(r2);
-                PE[NP][0] = dx; PE[NP][1] = dy; PE[NP][2] = dz;
-                PK[NP][0] = (float)(dx / L); PK[NP][1] = (float)(dy / L); PK[NP][2] = (float)(dz / L);
-                NP++;
-                second += 2.0 * dz * dz / L;
-            }
+    NE = 0;
+    for (int pass = 0; pass < 2; pass++)
+        for (int dx = 0; dx <= R; dx++)
+            for (int dy = -R; dy <= R; dy++)
+                for (int dz = -R; dz <= R; dz++) {
+                    int pos = dx > 0 || (dx == 0 && (dy > 0 || (dy == 0 && dz > 0)));
+                    double r2 = dx * dx + dy * dy + dz * dz;
+                    if (!pos || !(r2 > lo && r2 <= hi)) continue;
+                    double L = sqrt(r2);
+                    int coupled = COUPLES && dz != 0 && (dx != 0 || dy != 0);
+                    if (pass == 0) second += 2.0 * dz * dz / L;
+                    if (coupled != (pass == 0) || (coupled && dz < 0)) continue;
+                    PE[NE][0] = dx; PE[NE][1] = dy; PE[NE][2] = dz;
+                    PK[NE][0] = (float)(dx / L); PK[NE][1] = (float)(dy / L); PK[NE][2] = (float)(dz / L);
+                    PC[NE++] = coupled;
+                }
     WSH = (4 * M_PI / 3) * SIG / second;
     int Rb = (int)floor(SIG / 2);
     NB = 0;
@@ -213,11 +218,13 @@ static node_fn variant(const char *s)
 
 int main(int argc, char **argv)
 {
-    if (argc != 11 || (strcmp(argv[10], "sym") && strcmp(argv[10], "asym"))) {
-        fprintf(stderr, "column <nz> <n*> <sigma> <tau> <g_x> <steps> <band> <band_mode> <inner_mode> <sym|asym>\n");
+    if (argc != 11 || (strcmp(argv[10], "sym") && strcmp(argv[10], "asym") && strcmp(argv[10], "couple"))) {
+        fprintf(stderr, "column <nz> <n*> <sigma> <tau> <g_x> <steps> <band> <band_mode> <inner_mode> "
+                        "<sym|asym|couple>\n");
         return 2;
     }
     QD_ASYM = !strcmp(argv[10], "asym");
+    COUPLES = !strcmp(argv[10], "couple");
     NZ = atoi(argv[1]);
     double nstar = atof(argv[2]);
     SIG = atof(argv[3]);

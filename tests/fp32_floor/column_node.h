@@ -1,7 +1,8 @@
 /* One node's shell sums, fields and collision with push streaming, in the
  * arithmetic of the FP32 tiled kernel: deviation fields, (+e, -e) pair weights
- * with the exact divided difference of the closure, accumulators in table
- * order, second-order forcing with the A-term.  Included by column.c once per
+ * with the exact divided difference of the closure, accumulators in the order of
+ * the entries (single pairs in table order, or mirror couples first, the
+ * kernel's), second-order forcing with the A-term.  Included by column.c once per
  * precision variant: TW is the type of the pair weights, accumulators and
  * forces, TC the type of the collision, FETCH the neighbour loader of type TW.
  * Q+ - Q- takes the kernel's form, odd under swapping the pair's ends bit for
@@ -11,25 +12,43 @@
         TW noff=(TW)NOFF, hoff=(TW)HOFF, hr = hoff + (TW)hb[z], s0 = (TW)1 - hr - hoff;
         TW me_dn=(TW)nudn[z], vx=(TW)nuv[0][z], vy=(TW)nuv[1][z], vz=(TW)nuv[2][z];
         TW Vx=0,Vy=0,Vz=0,Wx=0,Wy=0,Wz=0,Sxx=0,Syy=0,Szz=0,Sxy=0,Sxz=0,Syz=0,t=0;
-        for(int m=0;m<NP;m++){
-            TW dnp,hp,vp[3],dnm,hm,vm[3]; FETCH(z+PE[m][2],&dnp,&hp,vp); FETCH(z-PE[m][2],&dnm,&hm,vm);
-            TW gnoff=(TW)noff, gs0=(TW)s0, ghp=(TW)hp, ghm=(TW)hm, gdnp=(TW)dnp, gdnm=(TW)dnm;
-            TW np=gnoff+gdnp, nm=gnoff+gdnm, sp=gs0-ghp, sm=gs0-ghm, spm=sp*sm, sp2=sp*sp, sm2=sm*sm;
-            TW rp=(TW)1/(sp2*sp), rm=(TW)1/(sm2*sm);
-            TW gp=fma(sp,rp,rp), gm=fma(sm,rm,rm);
-            TW gd=(ghp-ghm)*((sp2+sm2)+fma(spm,sp+sm,spm))*(rp*rm);
-            TW qp=gp*np, qm=gm*nm, qd=QD_ASYM ? fma(gp,gdnp-gdnm,gd*nm) : (TW)0.5*fma(gp+gm,gdnp-gdnm,gd*(np+nm));
+        for(int m=0;m<NE;m++){
+            /* terms of the entry's pair or, in a couple, of its two pairs */
+            TW dx[2],dy[2],dz[2],ks[2],qd[2],tq[2];
+            for(int h=0;h<=PC[m];h++){
+                int ez=h?-PE[m][2]:PE[m][2];
+                TW dnp,hp,vp[3],dnm,hm,vm[3]; FETCH(z+ez,&dnp,&hp,vp); FETCH(z-ez,&dnm,&hm,vm);
+                TW gnoff=(TW)noff, gs0=(TW)s0, ghp=(TW)hp, ghm=(TW)hm, gdnp=(TW)dnp, gdnm=(TW)dnm;
+                TW np=gnoff+gdnp, nm=gnoff+gdnm, sp=gs0-ghp, sm=gs0-ghm, spm=sp*sm, sp2=sp*sp, sm2=sm*sm;
+                TW rp=(TW)1/(sp2*sp), rm=(TW)1/(sm2*sm);
+                TW gp=fma(sp,rp,rp), gm=fma(sm,rm,rm);
+                TW gd=(ghp-ghm)*((sp2+sm2)+fma(spm,sp+sm,spm))*(rp*rm);
+                TW qp=gp*np, qm=gm*nm;
+                qd[h]=QD_ASYM ? fma(gp,gdnp-gdnm,gd*nm) : (TW)0.5*fma(gp+gm,gdnp-gdnm,gd*(np+nm));
+                TW kx=(TW)PK[m][0], ky=(TW)PK[m][1], kz=(TW)(h?-PK[m][2]:PK[m][2]);
+                TW px=qp*(TW)vp[0],py=qp*(TW)vp[1],pz=qp*(TW)vp[2];
+                dx[h]=fma(-qm,(TW)vm[0],px);dy[h]=fma(-qm,(TW)vm[1],py);dz[h]=fma(-qm,(TW)vm[2],pz);
+                TW ex=fma(qm,(TW)vm[0],px),ey=fma(qm,(TW)vm[1],py),ez_=fma(qm,(TW)vm[2],pz);
+                tq[h]=qp+qm;
+                TW sx=fma(-tq[h],(TW)vx,ex),sy=fma(-tq[h],(TW)vy,ey),sz=fma(-tq[h],(TW)vz,ez_);
+                ks[h]=fma(kx,sx,fma(ky,sy,kz*sz));
+            }
             TW kx=(TW)PK[m][0], ky=(TW)PK[m][1], kz=(TW)PK[m][2];
-            TW px=qp*(TW)vp[0],py=qp*(TW)vp[1],pz=qp*(TW)vp[2];
-            TW dx=fma(-qm,(TW)vm[0],px),dy=fma(-qm,(TW)vm[1],py),dz=fma(-qm,(TW)vm[2],pz);
-            TW ex=fma(qm,(TW)vm[0],px),ey=fma(qm,(TW)vm[1],py),ez=fma(qm,(TW)vm[2],pz);
-            TW tq=qp+qm; t+=tq;
-            TW sx=fma(-tq,(TW)vx,ex),sy=fma(-tq,(TW)vy,ey),sz=fma(-tq,(TW)vz,ez);
-            Vx=fma((TW)kx,(TW)qd,Vx);Vy=fma((TW)ky,(TW)qd,Vy);Vz=fma((TW)kz,(TW)qd,Vz);
-            TW ks=fma(kx,sx,fma(ky,sy,kz*sz));
-            Wx=fma((TW)kx,(TW)ks,Wx);Wy=fma((TW)ky,(TW)ks,Wy);Wz=fma((TW)kz,(TW)ks,Wz);
-            Sxx=fma((TW)kx,(TW)dx,Sxx);Syy=fma((TW)ky,(TW)dy,Syy);Szz=fma((TW)kz,(TW)dz,Szz);
-            Sxy=fma((TW)ky,(TW)dx,fma((TW)kx,(TW)dy,Sxy));Sxz=fma((TW)kz,(TW)dx,fma((TW)kx,(TW)dz,Sxz));Syz=fma((TW)kz,(TW)dy,fma((TW)ky,(TW)dz,Syz));
+            if(PC[m]){
+                t+=tq[0]+tq[1];
+                TW vs=qd[0]+qd[1], vd=qd[0]-qd[1], ws=ks[0]+ks[1], wd=ks[0]-ks[1];
+                Vx=fma(kx,vs,Vx);Vy=fma(ky,vs,Vy);Vz=fma(kz,vd,Vz);
+                Wx=fma(kx,ws,Wx);Wy=fma(ky,ws,Wy);Wz=fma(kz,wd,Wz);
+                TW xs=dx[0]+dx[1],ys=dy[0]+dy[1],zs=dz[0]+dz[1],xd=dx[0]-dx[1],yd=dy[0]-dy[1],zd=dz[0]-dz[1];
+                Sxx=fma(kx,xs,Sxx);Syy=fma(ky,ys,Syy);Szz=fma(kz,zd,Szz);
+                Sxy=fma(ky,xs,fma(kx,ys,Sxy));Sxz=fma(kz,xd,fma(kx,zs,Sxz));Syz=fma(kz,yd,fma(ky,zs,Syz));
+            } else {
+                t+=tq[0];
+                Vx=fma(kx,qd[0],Vx);Vy=fma(ky,qd[0],Vy);Vz=fma(kz,qd[0],Vz);
+                Wx=fma(kx,ks[0],Wx);Wy=fma(ky,ks[0],Wy);Wz=fma(kz,ks[0],Wz);
+                Sxx=fma(kx,dx[0],Sxx);Syy=fma(ky,dy[0],Syy);Szz=fma(kz,dz[0],Szz);
+                Sxy=fma(ky,dx[0],fma(kx,dy[0],Sxy));Sxz=fma(kz,dx[0],fma(kx,dz[0],Sxz));Syz=fma(kz,dy[0],fma(ky,dz[0],Syz));
+            }
         }
         TW n = (TW)noff + (TW)me_dn, wh=(TW)0.5*(TW)WSH, mf=-(TW)(1.0/3)*(TW)SIG2*wh*n, vi=(TW)BETA*wh*n, ovx=(TW)vx, ovy=(TW)vy, ovz=(TW)vz;
         TW Cx=mf*(TW)Vx+vi*(TW)Wx, Cy=mf*(TW)Vy+vi*(TW)Wy, Cz=mf*(TW)Vz+vi*(TW)Wz;
