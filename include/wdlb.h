@@ -144,9 +144,8 @@ typedef struct {
                                  wdlb_batch_step call in which each pore's phases
                                  follow one another without device-wide barriers
                                  (used where every pore runs the tiled sigma-4 kernel
-                                 on 8 x 8 x 4 bricks, which such a batch's pores take
-                                 unless tile forces a shape; else the default).  Both
-                                 give bitwise the same results                       */
+                                 on 8 x 8 x 4 bricks, else the default).  Both give
+                                 bitwise the same results                            */
     int32_t collision;        /* arithmetic of the collision and push (step 3 of
                                  Sec. 5, Eq. SMDB) with FP32 storage:
                                  WDLB_COLLISION_FP32 (default) FP32; with walls

@@ -535,19 +535,19 @@ bool tiled_applies(wdlb_lattice lat, double sigma, const wdlb_options &o)
            lat.nx >= 8 && lat.ny >= 8;
 }
 
-// Built-in choice when no probe runs, the probe's winners: the 512-thread shape
-// for sigma 6 (one 160 KB block per SM), 8^3 bricks for sigma 3 (three 55 KB
-// blocks per SM) and for the compact shell at sigma 4, 8 x 8 x 4 bricks for the
-// full shell at sigma 4 (three 61 KB blocks per SM).  Shell kernel of the three
-// shapes, ms, 128^3 box / 152 x 152 x 41 slit: sigma 3 full 0.290 0.331 0.298 /
-// 0.135 0.158 0.144, compact 0.155 0.211 0.172 / 0.077 0.102 0.086; sigma 4 full
-// 0.501 0.573 0.497 / 0.241 0.274 0.233, compact 0.199 0.262 0.211 / 0.103 0.133
-// 0.106; sigma 6 full 1.301 1.095 1.362, compact 0.304 0.267 0.398.
-int tile_builtin(int s2, int rule)
+// Built-in choice when no probe runs: the 512-thread shape for sigma 6 (one 160 KB
+// block per SM), 8 x 8 x 4 bricks for sigma 4 (three 61 KB blocks per SM), 8^3
+// bricks for sigma 3 (three 55 KB blocks per SM).  They are the probe's winners,
+// but for the compact shell at sigma 4, where 8^3 bricks are 2 to 6 % faster and
+// a probe takes them: unprobed, its pores keep the shape that the persistent kernel
+// serves.  Shell kernel of the three shapes, ms, 128^3 box / 152 x 152 x 41 slit:
+// sigma 3 full 0.290 0.331 0.298 / 0.135 0.158 0.144, compact 0.155 0.211 0.172 /
+// 0.077 0.102 0.086; sigma 4 full 0.501 0.573 0.497 / 0.241 0.274 0.233, compact
+// 0.199 0.262 0.211 / 0.103 0.133 0.106; sigma 6 full 1.301 1.095 1.362, compact
+// 0.304 0.267 0.398.
+int tile_builtin(int s2)
 {
-    return s2 == 12                                ? WDLB_TILE_8x8x8_WIDE
-           : s2 == 8 && rule == WDLB_SHELL_FULL ? WDLB_TILE_8x8x4
-                                                   : WDLB_TILE_8x8x8;
+    return s2 == 12 ? WDLB_TILE_8x8x8_WIDE : (s2 == 8 ? WDLB_TILE_8x8x4 : WDLB_TILE_8x8x8);
 }
 
 // Time each shape's shell kernel on a scratch lattice of the key: nz as
@@ -597,7 +597,7 @@ int choose_tile(wdlb_lattice lat, double sigma, int32_t walls, const wdlb_option
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     auto it = g_tune.find(key);
     if (it != g_tune.end()) return it->second;
-    int v = tile_builtin(key.s2, o.shell_rule);
+    int v = tile_builtin(key.s2);
     // The built-in shape stays unless another is faster by more than the probe's
     // noise (2 %): two shapes within it would be drawn at random per nz, and the
     // pores of one batch would fall into several shell launches.
@@ -1610,8 +1610,6 @@ wdlb_status wdlb_batch_add(wdlb_batch *b, const wdlb_pore_desc *d, const double 
     o.workspace = b->pool + off;
     o.workspace_bytes = need;
     o.stream = b->stream;
-    // the persistent kernel serves one shape (do_flow_ok); every shape gives the same bits
-    if (o.persistent && o.tile < 0 && two_sigma(d->sigma) == 8) o.tile = WDLB_TILE_8x8x4;
     wdlb_ctx *c = nullptr;
     st = wdlb_create(d->lat, d->sigma, d->walls, d->tau, d->g, &o, &c);
     if (st != WDLB_OK) {
