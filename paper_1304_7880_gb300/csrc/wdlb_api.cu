@@ -275,9 +275,11 @@ wdlb_status check_status_word(wdlb_ctx *ctx)
 // / 3 684 on 64 of them, 156 / 166 on 36 864.  Does not: sigma 8 compact FP32 (21)
 // 18.6 / 12.4 on 16 384 nodes, but 232 / 292 on 64 of them; sigma 1.5 full FP32
 // (13) 14 / 10 and 169 / 215; sigma 3 compact FP64 (13) 2 771 / 2 933 on 64.
-int split_shell(int storage, int npair, long long N)
+// Without interactions there is no sum to split (FP64 64^3 328 / 427 per step).
+int split_shell(const wdlb_options &o, int npair, long long N)
 {
-    return npair >= 31 || (storage == WDLB_STORE_F64 && npair >= 19 && N <= 24576) ? 1 : 0;
+    if (!o.interactions) return 0;
+    return npair >= 31 || (o.storage == WDLB_STORE_F64 && npair >= 19 && N <= 24576) ? 1 : 0;
 }
 
 void set_params(wdlb_ctx *ctx)
@@ -315,7 +317,7 @@ void set_params(wdlb_ctx *ctx)
     p.tiled = 0;
     p.shell_r = 0;
     for (int c : ctx->tab.shell) p.shell_r = std::max(p.shell_r, std::abs(c));
-    p.split = split_shell(ctx->opt.storage, p.nshell / 2, ctx->N);
+    p.split = split_shell(ctx->opt, p.nshell / 2, ctx->N);
     p.ball_r = 0;
     for (size_t m = 0; m < ctx->tab.ball.size(); m++) p.ball_r = std::max(p.ball_r, std::abs(ctx->tab.ball[m]));
     const size_t tsize = ctx->opt.storage == WDLB_STORE_F64 ? sizeof(double) : sizeof(float);
@@ -678,7 +680,7 @@ wdlb_status wdlb_create(wdlb_lattice lat, double sigma, int32_t walls, double ta
     build_shell_rule(sigma, o.shell_rule, ctx->tab.shell, ctx->tab.wvec);
     // couples need one weight for all pairs; the unsplit generic kernel keeps the table's order
     if (o.shell_rule == WDLB_SHELL_FULL && o.storage != WDLB_STORE_F16 &&
-        split_shell(o.storage, (int)ctx->tab.shell.size() / 6, ctx->N))
+        split_shell(o, (int)ctx->tab.shell.size() / 6, ctx->N))
         ctx->tab.ncouple = order_couples(ctx->tab.shell);
     ctx->tab.wshell = o.shell_rule == WDLB_SHELL_COMPACT ? 1.0 : ctx->tab.wvec[0];
     ctx->L = &launchers_for(o.storage, o.collision);

@@ -90,6 +90,24 @@ def test_generic_forms_match_the_oracle(w, oracle_mod, lat, sigma, walls, storag
     w.wdlb_destroy(ctx)
 
 
+@pytest.mark.parametrize("storage,closure", [("f64", "CS"), ("f32", "PY")])
+def test_without_interactions_nothing_is_split(w, oracle_mod, storage, closure):
+    lat = (9, 8, 23)
+    n, u = synth.uniform_with_noise(*lat, 0.3 / 64, 2e-2, 7, True)
+    ctx = w.wdlb_create(lat, 4.0, True, 1.0, (1e-5, 0.0, 0.0), storage=storage, closure=closure, interactions=False)
+    w.wdlb_init_fields(ctx, n, u)
+    assert w.wdlb_shell_info(ctx) == (False, False)
+    o = oracle_mod.Oracle(*lat, True, 4.0, 1.0, (1e-5, 0.0, 0.0), closure=closure, interactions=False)
+    o.init(n, u)
+    w.wdlb_step(ctx, 4)
+    o.step(4)
+    (n_g, u_g), (n_o, u_o) = w.wdlb_moments(ctx), o.moments()
+    tn, tu = TOL[storage]
+    np.testing.assert_allclose(n_g[1:-1], n_o[1:-1], rtol=tn)
+    np.testing.assert_allclose(u_g[:, 1:-1], u_o[:, 1:-1], rtol=0, atol=tu * np.abs(u_o[:, 1:-1]).max())
+    w.wdlb_destroy(ctx)
+
+
 def test_batch_of_split_and_unsplit_groups(w):
     b = w.wdlb_batch_create(3, 64 << 20, storage="f32")
     for lat, sigma in (((9, 8, 25), 8.0), ((8, 8, 17), 1.5), ((9, 11, 25), 4.0)):
