@@ -275,7 +275,8 @@ wdlb_status check_status_word(wdlb_ctx *ctx)
 // / 3 684 on 64 of them, 156 / 166 on 36 864.  Does not: sigma 8 compact FP32 (21)
 // 18.6 / 12.4 on 16 384 nodes, but 232 / 292 on 64 of them; sigma 1.5 full FP32
 // (13) 14 / 10 and 169 / 215; sigma 3 compact FP64 (13) 2 771 / 2 933 on 64.
-// Without interactions there is no sum to split (FP64 64^3 328 / 427 per step).
+// Without interactions there is no sum to split: 64^3 in FP64 takes 330 us per step
+// unsplit and 427 split.
 int split_shell(const wdlb_options &o, int npair, long long N)
 {
     if (!o.interactions) return 0;
@@ -601,12 +602,12 @@ int choose_tile(wdlb_lattice lat, double sigma, int32_t walls, const wdlb_option
     if (it != g_tune.end()) return it->second;
     int v = tile_builtin(key.s2);
     // The built-in shape stays unless another is faster by more than the probe's
-    // noise (2 %): two shapes within it would be drawn at random per nz, and the
-    // pores of one batch would fall into several shell launches.
+    // noise (below 1 %): two shapes within it would be drawn at random per nz, and
+    // the pores of one batch would fall into several shell launches.
     if (o.autotune) {
         int b = -1;
         double ms[3];
-        if (probe_tiles(lat, sigma, walls, o, &b, ms) == WDLB_OK && !(ms[b] > 0.98 * ms[v])) v = b;
+        if (probe_tiles(lat, sigma, walls, o, &b, ms) == WDLB_OK && !(ms[b] > 0.99 * ms[v])) v = b;
     }
     g_tune[key] = v;
     return v;

@@ -672,7 +672,8 @@ __device__ __forceinline__ void collide_push(const KParams &p, const KBufs<S, T>
         // driven slit by up to 6e-5 of max|u_x|.  The correction carries no mass
         // (sum_q w_q c_q = 0).  The wall-normal component, which the walls take
         // up, is left as it is: correcting it too raised the density error of
-        // the converged slit at n* 0.3 from 1.1e-7 to 8.3e-7.
+        // the converged slit at n* 0.3 from 1.1e-7 to 8.3e-7 (pairs summed one by
+        // one; 8.3e-8 with the couples).
         dwf Mx = dw_from(0.f), My = dw_from(0.f);
 #pragma unroll
         for (int q = 0; q < NQ; q++) {
@@ -927,7 +928,8 @@ __device__ __forceinline__ void shell_body(const KParams &p, const KBufs<S, type
 // ---------------------------------------------------------------------------
 // Split form of shell_body: a block of kSplit warps serves 32 nodes, lane l of
 // every warp the same node, and warp k sums the couples (then the pairs left
-// over) k, k + kSplit, ... of the table; warp 0 adds the partial sums in warp order and runs the collision.
+// over) k, k + kSplit, ... of the table; warp 0 adds the partial sums in warp
+// order and runs the collision.
 // Unsplit, the kernel is bound by each warp's own chain of loads and sums (FP32:
 // 381 pairs at sigma 8, ~400 instructions each) or by the FP64 pipe of the few
 // SMs that hold a block (two lanes a clock), so a lattice of few blocks leaves
@@ -936,12 +938,12 @@ __device__ __forceinline__ void shell_body(const KParams &p, const KBufs<S, type
 // component (2 R + 1 per axis) into shared memory; beyond a wall they point at
 // the solid plane z = 0, whose nu and hb hold the n = 0 state, so a neighbour's
 // index is the sum of three words with no test.  A couple takes one table entry:
-// its second pair is the first with z negated (sigma 8 on 8 x 8 x 256 41.2 ->
-// 31.1 us, 96^3 1 602 -> 1 238).  Shell kernel, unsplit with modulo wraps and now:
-// sigma 8 on 8 x 8 x 256 (FP32) 256.8 -> 31.1 us, bound by the latency of its
-// dependent loads (3.4 warps per scheduler); the 8 x 8 x 41 slit in FP64 547 -> 74
-// us, a 45 x 38 x 51 box in FP64 1 633 -> 1 005, bound by the FP64 pipe (about 55
-// operations per pair, two lanes per clock and SM).
+// its second pair is the first with z negated (sigma 8 on 8 x 8 x 256 37.4 ->
+// 33.3 us).  Shell kernel, unsplit with modulo wraps and now: sigma 8 on 8 x 8 x
+// 256 (FP32) 256.8 -> 33.3 us, bound by the latency of its dependent loads (3.4
+// warps per scheduler); the 8 x 8 x 41 slit in FP64 547 -> 86 us, a 45 x 38 x 51
+// box in FP64 1 633 -> 1 122, bound by the FP64 pipe (about 60 operations per
+// pair, two lanes per clock and SM).
 // ---------------------------------------------------------------------------
 constexpr int kSplit = 4;   // (eight: 96^3 at sigma 8 1 607 -> 2 149 us, FP64 45 x 38 x 51 1 055 -> 1 369)
 
