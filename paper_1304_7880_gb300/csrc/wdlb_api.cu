@@ -680,7 +680,8 @@ wdlb_status wdlb_create(wdlb_lattice lat, double sigma, int32_t walls, double ta
     build_ball(sigma, ctx->tab.ball);
     build_shell_rule(sigma, o.shell_rule, ctx->tab.shell, ctx->tab.wvec);
     // couples need one weight for all pairs; the unsplit generic kernel keeps the table's order
-    if (o.shell_rule == WDLB_SHELL_FULL && o.storage != WDLB_STORE_F16 &&
+    if (o.shell_rule == WDLB_SHELL_FULL &&
+        sums_couples(o.storage == WDLB_STORE_F16, o.collision == WDLB_COLLISION_DW) &&
         split_shell(o, (int)ctx->tab.shell.size() / 6, ctx->N))
         ctx->tab.ncouple = order_couples(ctx->tab.shell);
     ctx->tab.wshell = o.shell_rule == WDLB_SHELL_COMPACT ? 1.0 : ctx->tab.wvec[0];

@@ -47,7 +47,7 @@ struct KParams {
     int nx, ny, nz, walls;   // walls: solid planes z = 0 and z = nz-1
     int N, Npad;             // node count, padded stride of per-node arrays
     int nshell, nball;
-    int ncouple;             // mirror couples at the head of the shell table (order_couples); 0: compact shell, FP16 storage
+    int ncouple;             // mirror couples at the head of the shell table (order_couples); 0: the table's order
     int closure, omega_mode, interactions;
     int s2;                  // 2 sigma if it is an integer, else 0 (selects a compiled shell)
     int tiled;               // 1: use the shared-memory tiled shell kernel
@@ -299,20 +299,14 @@ struct Store<__half> {
 };
 
 // Whether the full shell's pairs are summed as mirror couples (order_couples).
-// FP16 storage keeps the table's order: it is for periodic boxes, where the
-// couples' exact zeros along the walls have no part, and the rounding of its
-// stored populations turns a last bit of the sums into 2e-4 of u (96^3, sigma 6,
-// ten steps), so that another order would change every result visibly for
-// nothing but speed (shell kernel there 0.494 ms as couples, 0.508 so).
-template <class S>
-constexpr bool sums_couples()
-{
-    return true;
-}
-template <>
-constexpr bool sums_couples<__half>()
-{
-    return false;
-}
+// Two options keep the table's order:
+// FP16 storage, which is for periodic boxes, where the couples' exact zeros along
+// the walls have no part: the rounding of its stored populations turns a last bit
+// of the sums into 2e-4 of u (96^3, sigma 6, ten steps), so that another order
+// would change every result visibly for nothing but speed (shell kernel there
+// 0.494 ms as couples, 0.508 so).
+// The double-word collision, the accuracy option: the converged 161-node slit at
+// n* 0.3 is 4.8e-6 off on u_x so and 9.3e-6 with couples (2 % faster).
+constexpr bool sums_couples(bool f16_storage, bool dw_collision) { return !f16_storage && !dw_collision; }
 
 }  // namespace wdlb

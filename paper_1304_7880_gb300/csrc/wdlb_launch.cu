@@ -179,7 +179,7 @@ bool compiled_table_matches()
     } else {
         double w = 0.0;
         build_shell(sigma, e, &w);
-        constexpr bool CPL = sums_couples<S>();
+        constexpr bool CPL = sums_couples(std::is_same<S, __half>::value, is_dw<A>::value);
         const tiled::ct::FullTable<S2, CPL> &T = tiled::ct::kFull<S2, CPL>;
         if ((CPL ? order_couples(e) : 0) != T.nc || (int)e.size() != 6 * (2 * T.nc + T.ns)) return false;
         constexpr int SX = tiled::TX + 2 * tiled::shell_radius(S2);

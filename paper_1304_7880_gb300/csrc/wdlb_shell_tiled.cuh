@@ -470,7 +470,7 @@ __device__ __forceinline__ void tiled_body(const KParams &p, const KBufs<S, floa
             // registers, so an address takes none; two couples per iteration for
             // sigma 3 and 4 (1, 3 and 4 measured 3, 1 and 1.5 % slower), one for
             // sigma 6.
-            constexpr bool CPL = sums_couples<S>();
+            constexpr bool CPL = sums_couples(std::is_same<S, __half>::value, is_dw<A>::value);
             constexpr int kUnroll = ROOMY ? 4 : S2 >= 12 ? 1 : CPL ? 2 : 3;
             if constexpr (!WT) {
                 constexpr int NC = ct::kFull<S2, CPL>.nc, NSI = ct::kFull<S2, CPL>.ns;
